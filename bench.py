@@ -41,7 +41,8 @@ if ROOT not in sys.path:
 METRIC = "MLUPS and % of HBM roofline per form at <=1e-3 rel-L2 vs FP64 oracle"
 UNIT = "MLUPS"
 WORKLOAD = dict(lattice="D3Q19", n=256, Re=100.0, Wi=1.0, beta=0.5, U0=0.02)
-KERNEL_SOURCES = ["paper_2506_13072_gb300/csrc/fvlb_kernels.cuh",
+KERNEL_SOURCES = ["paper_2506_13072_gb300/csrc/fvlb_fused.cuh",
+                  "paper_2506_13072_gb300/csrc/fvlb_kernels.cuh",
                   "paper_2506_13072_gb300/csrc/fvlb_lattice.cuh",
                   "paper_2506_13072_gb300/csrc/fvlb_launch.cuh"]
 
@@ -273,25 +274,16 @@ def kernel_label(lattice: str, precision: str) -> str:
     """The fused-step kernel instance the library launches for this workload."""
     S = {"fp64": "double", "fp32": "float", "fp16_dev": "__half", "bf16_dev": "__nv_bfloat16",
          "fp16_dev_sr": "half_sr", "bf16_dev_sr": "bf16_sr"}[precision]
-    minb = 1 if precision == "fp64" else 2
+    wide, half = precision == "fp64", precision not in ("fp64", "fp32")
     if lattice == "d2q9":
-        if precision == "fp64":
-            return (f"k_step_fused<D2Q9,double,GX=4,TY=1,MINB=1,periodic> "
-                    f"(128 nodes x 3 stress components per block, in-warp halo fill)")
-        nfw = 5 if precision == "fp32" else 4
-        return (f"k_step_fused<D2Q9,{S},GX=4,TY=1,MINB=2,periodic,fill warps> "
-                f"(128 nodes x 3 stress components + {nfw} halo fill warps per block, "
-                f"bulk tensor copies into the stage)")
-    if precision == "fp32":
-        return (f"k_step_fused<D3Q19,float,GX=1,TY=1,MINB=2,periodic,fill warps,XN=2> "
-                f"(64 nodes x 6 stress components + 7 halo fill warps per block, "
-                f"bulk tensor copies into the stage)")
-    if precision == "fp64":
-        return (f"k_step_fused<D3Q19,double,GX=1,TY=1,MINB=1,periodic,fill warps> "
-                f"(32 nodes x 6 stress components + 4 halo fill warps per block)")
-    return (f"k_step_fused<D3Q19,{S},GX=1,TY=1,MINB=2,periodic,fill warps,XN=2> "
-            f"(64 nodes x 6 stress components + 4 halo fill warps per block, "
-            f"bulk tensor copies into the stage)")
+        gx, kg, minb = (2, 1, 3) if wide else ((4, 1, 4) if half else (4, 1, 2))
+        slots, lat = 32 * gx + 2, "D2Q9"
+    else:
+        gx, kg, minb = (1, 2, 2) if wide else ((2, 2, 3) if half else (2, 2, 2))
+        slots, lat = 3 * (32 * gx + 2), "D3Q19"
+    nfw = -(-(slots // 2 + (3 if lat == "D3Q19" else 1) if half else slots) // 32)
+    return (f"k_step_fused<{lat},{S},GX={gx},KG={kg},MINB={minb},periodic> ({32 * gx} nodes x {kg} "
+            f"thread(s) per node + {nfw} halo fill warps per block, bulk tensor copies into the stage)")
 
 
 def config_dict(args=None, note=""):

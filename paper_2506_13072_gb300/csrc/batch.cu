@@ -20,6 +20,8 @@ namespace fvlb {
 #define FVLB_EXTERN_BATCH(S)                                                             \
   extern template cudaError_t batch_step_impl<S>(const BatchLaunch&);                    \
   extern template int batch_occupancy_impl<S>(int);                                      \
+  extern template void batch_maps_impl<S>(StageMaps*, int, const void*, const void*,     \
+                                          const void*, long long);                                      \
   extern template void batch_inst_fill_impl<S>(void*, int, int, int, long long, double,  \
                                                double, double, double, int, const double*, \
                                                double, const void*, long long, long long,  \
@@ -46,6 +48,16 @@ int batch_occupancy(int storage, int gx) {
     case kFP32: return batch_occupancy_impl<float>(gx);
     case kFP16Dev: return batch_occupancy_impl<__half>(gx);
     default: return batch_occupancy_impl<__nv_bfloat16>(gx);
+  }
+}
+
+void batch_maps(int storage, StageMaps* m, int gx, const void* f, const void* h, const void* chi,
+                long long pitch) {
+  switch (storage) {
+    case kFP64: batch_maps_impl<double>(m, gx, f, h, chi, pitch); break;
+    case kFP32: batch_maps_impl<float>(m, gx, f, h, chi, pitch); break;
+    case kFP16Dev: batch_maps_impl<__half>(m, gx, f, h, chi, pitch); break;
+    default: batch_maps_impl<__nv_bfloat16>(m, gx, f, h, chi, pitch); break;
   }
 }
 
@@ -105,6 +117,7 @@ struct fvlb_batch_s {
   void* tables = nullptr;
   void* inst = nullptr;
   void* tiles = nullptr;
+  StageMaps* maps = nullptr;  // [parity][instance] of the current tile width
   int tiles_cap = 0;
   long long* tdev = nullptr;
   double* fbuf = nullptr;
@@ -112,7 +125,7 @@ struct fvlb_batch_s {
   long long t = 0;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  int gx = 4, mchunk = 16, ntiles = 0, blocks = 0;
+  int gx = 4, mchunk = 16, ntiles = 0, blocks = 0, maps_gx = 0;
   bool tuned = false;
   double tuned_ms = 0.0;
   cudaGraphExec_t graph = nullptr;
@@ -178,6 +191,23 @@ int upload_tiles(fvlb_batch_t b, int gx, int mchunk) {
                                   cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return bfail(b, FVLB_ECUDA, std::string("tile upload: ") + cudaGetErrorString(e));
+  if (gx != b->maps_gx) {
+    // the tensor maps of both parities for tiles of this width
+    std::vector<StageMaps> mp(2 * (size_t)b->count);
+    const size_t sb = sbytes(b->storage), xb = xbytes(b->storage);
+    for (int q = 0; q < 2; ++q)
+      for (int i = 0; i < b->count; ++i)
+        batch_maps(b->storage, &mp[(size_t)q * b->count + i], gx,
+                   static_cast<char*>(q ? b->fB : b->fA) + sb * b->f_off[i],
+                   static_cast<char*>(q ? b->hB : b->hA) + sb * b->h_off[i],
+                   static_cast<char*>(b->chi) + xb * b->chi_off[i], b->pitch[i]);
+    e = cudaMemcpyAsync(b->maps, mp.data(), mp.size() * sizeof(StageMaps), cudaMemcpyHostToDevice,
+                        b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    if (e != cudaSuccess)
+      return bfail(b, FVLB_ECUDA, std::string("tensor map upload: ") + cudaGetErrorString(e));
+    b->maps_gx = gx;
+  }
   b->gx = gx;
   b->mchunk = mchunk;
   b->ntiles = (int)tl.size();
@@ -210,6 +240,7 @@ BatchLaunch make_launch(fvlb_batch_t b) {
   d.tstep = b->tdev;
   d.mchunk = b->mchunk;
   d.blocks = b->blocks;
+  d.maps = b->maps + (size_t)b->parity * b->count;
   d.stream = b->stream;
   return d;
 }
@@ -236,6 +267,7 @@ int build_graph(fvlb_batch_t b) {
   for (int q = 0; q < 2; ++q) {
     BatchLaunch d = make_launch(b);
     d.parity = b->parity ^ q;
+    d.maps = b->maps + (size_t)d.parity * b->count;
     d.first = 0;
     if (e == cudaSuccess) e = batch_step(d);
     if (e == cudaSuccess) e = batch_advance(b->tdev, b->stream);
@@ -392,9 +424,10 @@ int fvlb_batch_create(fvlb_batch_t* out, int lattice, int count, const fvlb_inst
   // the finest shape (32 nodes x 8 rows) has the most tiles
   b->tiles_cap = (int)make_tiles(b, 1, 8).size();
   b->tiles = balloc(b, sizeof(BatchTile) * b->tiles_cap);
+  b->maps = static_cast<StageMaps*>(balloc(b, sizeof(StageMaps) * 2 * (size_t)count));
   b->tdev = static_cast<long long*>(balloc(b, sizeof(long long)));
   b->fbuf = static_cast<double*>(balloc(b, sizeof(double) * 6 * b->Nmax));
-  if (!b->fA || !b->fB || !b->hA || !b->hB || !b->chi || !b->inst || !b->tiles || !b->tdev ||
+  if (!b->fA || !b->fB || !b->hA || !b->hB || !b->chi || !b->inst || !b->tiles || !b->maps || !b->tdev ||
       !b->fbuf || (b->tab_total && !b->tables)) {
     bfree_all(b);
     cudaStreamDestroy(b->stream);

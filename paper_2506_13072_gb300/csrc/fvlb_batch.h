@@ -20,6 +20,7 @@ struct BatchLaunch {
   const long long* tstep;
   int mchunk;
   int blocks;
+  const void* maps;   // device array of StageMaps, one per instance (null: no bulk copies)
   cudaStream_t stream;
 };
 

@@ -7,30 +7,24 @@
 
 namespace fvlb {
 
-// Register budgets: GX groups of 32 nodes x 3 components = 96 GX threads,
-// MINB blocks per SM.
-template <int GX>
-struct BatchMinB {
-  static constexpr int value = GX == 4 ? 2 : (GX == 2 ? 4 : 8);
-};
-
-// dynamic shared memory of the batched kernel's tile (0: static)
+// Resident blocks per SM: at most 18 warps, so that the loop over tiles keeps
+// its state in registers (FP64: as its stage buffers allow).
 template <class S, int GX>
-constexpr size_t batch_dyn() {
-  return TileCfg<D2Q9, S, GX, 1, false, false, 1>::kDynamicBytes;
-}
+struct BatchMinB {
+  static constexpr int KG = sizeof(S) == 8 ? 3 : 1;
+  static constexpr int value = sizeof(S) == 8 ? 4 / GX : 18 * 32 / FusedShape<D2Q9, S, GX, KG>::NT;
+};
+template <class S, int GX>
+using BatchCfg = TileCfg<D2Q9, S, GX, BatchMinB<S, GX>::KG, BatchMinB<S, GX>::value, true, false>;
 
 template <class S, int GX>
 cudaError_t batch_launch_gx(const BatchLaunch& d) {
-  constexpr int MINB = BatchMinB<GX>::value;
-  constexpr int NT = FusedShape<D2Q9, GX, 1, false>::NT;
-  constexpr size_t dyn = batch_dyn<S, GX>();
+  constexpr int NT = FusedShape<D2Q9, S, GX, BatchMinB<S, GX>::KG>::NT;
+  constexpr size_t dyn = sizeof(typename BatchCfg<S, GX>::Smem);
   using X = typename Store<S>::X;
-  auto kern = k_step_batched<D2Q9, S, GX, MINB>;
-  if constexpr (dyn > 0) {
-    const cudaError_t e = allow_dynamic_smem(kern, dyn);
-    if (e != cudaSuccess) return e;
-  }
+  auto kern = k_step_batched<D2Q9, S, GX, BatchMinB<S, GX>::KG, BatchMinB<S, GX>::value>;
+  const cudaError_t e = allow_dynamic_smem(kern, dyn);
+  if (e != cudaSuccess) return e;
   int blocks = d.blocks;
   if (blocks <= 0) {
     int dev = 0, sms = 1, per = 1;
@@ -42,7 +36,8 @@ cudaError_t batch_launch_gx(const BatchLaunch& d) {
   kern<<<blocks, NT, dyn, d.stream>>>(
       static_cast<const BatchInst<S>*>(d.inst), static_cast<const BatchTile*>(d.tiles),
       d.ntiles, static_cast<S*>(d.fA), static_cast<S*>(d.fB), static_cast<S*>(d.hA),
-      static_cast<S*>(d.hB), static_cast<X*>(d.chi), d.parity, d.first, d.tstep, d.mchunk);
+      static_cast<S*>(d.hB), static_cast<X*>(d.chi), d.parity, d.first, d.tstep, d.mchunk,
+      static_cast<const StageMaps*>(d.maps));
   return cudaGetLastError();
 }
 
@@ -58,13 +53,11 @@ cudaError_t batch_step_impl(const BatchLaunch& d) {
 
 template <class S, int GX>
 int batch_occupancy_gx() {
-  auto kern = k_step_batched<D2Q9, S, GX, BatchMinB<GX>::value>;
-  constexpr size_t dyn = batch_dyn<S, GX>();
-  if constexpr (dyn > 0) {
-    if (allow_dynamic_smem(kern, dyn) != cudaSuccess) return 0;
-  }
+  auto kern = k_step_batched<D2Q9, S, GX, BatchMinB<S, GX>::KG, BatchMinB<S, GX>::value>;
+  constexpr size_t dyn = sizeof(typename BatchCfg<S, GX>::Smem);
+  if (allow_dynamic_smem(kern, dyn) != cudaSuccess) return 0;
   int per = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, FusedShape<D2Q9, GX, 1, false>::NT, dyn);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, FusedShape<D2Q9, S, GX, BatchMinB<S, GX>::KG>::NT, dyn);
   return per;
 }
 
@@ -75,6 +68,13 @@ int batch_occupancy_impl(int gx) {
     case 2: return batch_occupancy_gx<S, 2>();
     default: return batch_occupancy_gx<S, 4>();
   }
+}
+
+template <class S>
+void batch_maps_impl(StageMaps* m, int gx, const void* f, const void* h, const void* chi,
+                     long long pitch) {
+  const int BX = gx == 1 ? BatchCfg<S, 1>::BX : (gx == 2 ? BatchCfg<S, 2>::BX : BatchCfg<S, 4>::BX);
+  *m = stage_maps<D2Q9, S>(f, h, chi, pitch, BX);
 }
 
 template <class S>

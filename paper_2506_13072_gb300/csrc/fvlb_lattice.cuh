@@ -587,21 +587,49 @@ __device__ __forceinline__ void body_force(const Phys<R>& ph, int x, int y,
   }
 }
 
+// mo = sum_{i != 0} c_i f_i (f_0 is not read).  FP64: opposite directions
+// enter through their difference, which up to three sums share: 21 additions
+// in 3D and 8 in 2D, where direction by direction takes 30 and 12.
+template <class L, class R, class T>
+__device__ __forceinline__ void momentum(const T (&f)[L::Q], R (&mo)[L::D]) {
+  if constexpr (std::is_same<R, double>::value) {
+    bool any[L::D] = {};
+#pragma unroll
+    for (int i = 1; i < L::Q; ++i) {
+      const bool lead = L::cx(i) != 0 ? L::cx(i) > 0 : (L::cy(i) != 0 ? L::cy(i) > 0 : L::cz(i) > 0);
+      if (!lead) continue;
+      const R d = R(f[i]) - R(f[L::opp(i)]);
+#pragma unroll
+      for (int a = 0; a < L::D; ++a) {
+        const int c = cc<L>(i, a);
+        if (c == 0) continue;
+        mo[a] = !any[a] ? (c == 1 ? d : -d) : (c == 1 ? mo[a] + d : mo[a] - d);
+        any[a] = true;
+      }
+    }
+  } else {
+#pragma unroll
+    for (int a = 0; a < L::D; ++a) {
+      R m = R(0);
+#pragma unroll
+      for (int i = 1; i < L::Q; ++i) {
+        const int c = cc<L>(i, a);
+        if (c == 1) m += R(f[i]);
+        else if (c == -1) m -= R(f[i]);
+      }
+      mo[a] = m;
+    }
+  }
+}
+
 // u = sum_{i != 0} c_i f_i + F / 2   (Sec. 2.2)
 template <class L, class R>
 __device__ __forceinline__ void velocity(const R (&f)[L::Q], const R F[3],
                                          R (&u)[L::D]) {
+  R mo[L::D];
+  momentum<L, R>(f, mo);
 #pragma unroll
-  for (int a = 0; a < L::D; ++a) {
-    R m = R(0);
-#pragma unroll
-    for (int i = 1; i < L::Q; ++i) {
-      const int c = cc<L>(i, a);
-      if (c == 1) m += f[i];
-      else if (c == -1) m -= f[i];
-    }
-    u[a] = m + R(0.5) * F[a];
-  }
+  for (int a = 0; a < L::D; ++a) u[a] = mo[a] + R(0.5) * F[a];
 }
 
 // f^B for a symmetric polymer stress (compact components t[C]).  This is
@@ -641,6 +669,65 @@ __device__ __forceinline__ R fB_dir(int i, const R (&t)[L::C], R inv_tau_f) {
     return v * inv_tau_f;
   }
 }
+
+// fB_dir over inv_tau_f in FP32 with its roundings fixed: the order and the
+// fused multiply-adds are written out, so that no compiler changes them.
+template <class L>
+__device__ __forceinline__ float fB_ordered(int i, const float (&t)[L::C]) {
+  if (L::D == 2) {
+    const float a = t[0], s = t[1], b = t[2];
+    const int x = L::cx(i), y = L::cy(i);
+    if (i == 0) return __fmul_rn(a + b, float(1.0 / 3.0));
+    if (y == 0) return __fmul_rn(__fmaf_rn(2.f, b, -a), float(1.0 / 6.0));
+    if (x == 0) return __fmul_rn(__fmaf_rn(2.f, a, -b), float(1.0 / 6.0));
+    return __fmul_rn(-__fmaf_rn(2.f, a + b, __fmul_rn(float(3 * x * y), s)), float(1.0 / 12.0));
+  } else {
+    const int c0 = L::cx(i), c1 = L::cy(i), c2 = L::cz(i);
+    const int n = c0 * c0 + c1 * c1 + c2 * c2;
+    if (n == 0) return __fmul_rn(t[0] + t[1] + t[2], float(5.0 / 21.0));
+    if (n == 1) {
+      const float taa = t[c0 != 0 ? 0 : (c1 != 0 ? 1 : 2)];
+      return __fmaf_rn(t[0] + t[1] + t[2] - taa, float(1.0 / 7.0), __fmul_rn(-taa, float(1.0 / 42.0)));
+    }
+    const int g = c0 == 0 ? 0 : (c1 == 0 ? 1 : 2);  // axis normal to the plane
+    const int a = g == 0 ? 1 : 0, b = g == 2 ? 1 : 2;
+    const int cab = cc<L>(i, a) * cc<L>(i, b);
+    return __fmaf_rn(-0.25f * float(cab), t[sym<L>(a, b)],
+                     __fmaf_rn(t[g], float(1.0 / 21.0), __fmul_rn(-(t[a] + t[b]), float(5.0 / 42.0))));
+  }
+}
+
+// fB_dir for all directions of one node, from terms that directions share
+// (the same least-norm solution): rest q0; along axis a q1 - T_a; in the
+// plane (a, b) with normal g q2 + T_g -+ s_g in 3D (- where c_a c_b = 1),
+// q2 -+ s_0 in 2D.  In tr t: tr/7 - t_a/6 and -5 tr/42 + t_g/6 -+ t_ab/4 in
+// 3D, tr/3 - t_a/2 and -tr/6 -+ t_xy/4 in 2D.
+template <class L, class R>
+struct FBTerms {
+  R q0, q1, q2, T[L::D], s[L::D];
+  __device__ __forceinline__ void set(const R (&t)[L::C], R k) {
+    if constexpr (L::D == 2) {
+      const R tr = (t[0] + t[2]) * k;
+      q0 = q1 = tr * R(1.0 / 3.0);
+      q2 = tr * R(-1.0 / 6.0);
+      const R h = k * R(0.5);
+      T[0] = t[0] * h;
+      T[1] = t[2] * h;
+      s[0] = s[1] = t[1] * (k * R(0.25));
+    } else {
+      const R tr = (t[0] + t[1] + t[2]) * k;
+      q0 = tr * R(5.0 / 21.0);
+      q1 = tr * R(1.0 / 7.0);
+      q2 = tr * R(-5.0 / 42.0);
+      const R h = k * R(1.0 / 6.0), r = k * R(0.25);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) T[a] = t[a] * h;
+      s[0] = t[5] * r;   // by the axis normal to the plane: yz, xz, xy
+      s[1] = t[4] * r;
+      s[2] = t[3] * r;
+    }
+  }
+};
 
 // (grad u)_{ab} = d_a u_b, chi = -(A - I)/lambda + A.grad u + (grad u)^T.A
 // in compact components (Sec. 2.3); Ad = A - I.

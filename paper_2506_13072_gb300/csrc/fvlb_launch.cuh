@@ -6,6 +6,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <cstdlib>
 #include <cstring>
@@ -19,13 +20,7 @@
 
 namespace fvlb {
 
-// Tile shapes of the fused step: GX x TY groups of 32 x-consecutive nodes
-// (a warp spans x, so every population load and store is one coalesced
-// 128-byte line, shifted by at most one element for the pushes), C threads
-// per node, optional fill warps (FW); MINB is the number of resident blocks
-// per SM the register allocation must allow.  The shapes below were the
-// fastest of those measured on GB300 (256^3 D3Q19, 2048^2 D2Q9).
-// Launch-shape overrides from the environment, for tuning sweeps.
+// An integer from the environment.
 inline int tune_int(const char* name, int dflt) {
   const char* v = std::getenv(name);
   return v && *v ? std::atoi(v) : dflt;
@@ -92,62 +87,43 @@ inline bool encode_map(CUtensorMap* m, CUtensorMapDataType t, int rank, const vo
              CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The tensor maps of a fused launch whose warps stage rows of BX nodes
-// (StageMaps in fvlb_kernels.cuh); `on` = 0 (the kernel's cp.async
-// staging) when a row start cannot lie on a 16-byte boundary, a buffer is
-// not 16-byte aligned, an encoding fails, or FVLB_STAGE_TMA=0.
+// The tensor maps of a fused launch whose stage holds BX nodes of every
+// array (StageMaps in fvlb_kernels.cuh); `on` = 0 (each lane copies its own
+// node) when a buffer is not 16-byte aligned, an encoding fails, or
+// FVLB_STAGE_TMA=0.
 template <class L, class S>
-StageMaps stage_maps(const StepDesc& d, int BX) {
+StageMaps stage_maps(const void* f, const void* h, const void* chi, long long pitch, int BX) {
   StageMaps m;
   std::memset(&m, 0, sizeof m);
   constexpr int Q = L::Q, C = L::C, D = L::D;
-  constexpr int NJ = (Q - C) / C + 1;
-  constexpr cuuint64_t es = sizeof(S);
+  constexpr cuuint64_t es = sizeof(S), xs = sizeof(typename Store<S>::X);
   if (tune_int("FVLB_STAGE_TMA", 1) == 0) return m;
-  if (((cuuint64_t)d.nx * es) % 16 != 0 || ((cuuint64_t)d.pitch * es) % 16 != 0) return m;
   auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  if (!aligned(d.f_in) || !aligned(d.h_in) || !aligned(d.chi)) return m;
-  const CUtensorMapDataType t =
-      es == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_UINT16;
-  const CUtensorMapDataType tf = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
-  const cuuint64_t P = (cuuint64_t)d.pitch;
+  if (!aligned(f) || !aligned(h) || !aligned(chi)) return m;
+  const CUtensorMapDataType tf = CU_TENSOR_MAP_DATA_TYPE_FLOAT32, td = CU_TENSOR_MAP_DATA_TYPE_FLOAT64;
+  const CUtensorMapDataType t = es == 8 ? td : (es == 4 ? tf : CU_TENSOR_MAP_DATA_TYPE_UINT16);
+  const cuuint64_t P = (cuuint64_t)pitch;
   const cuuint32_t bx = (cuuint32_t)BX;
   bool ok = true;
-  {
-    const cuuint64_t dims[2] = {P, (cuuint64_t)C * Q}, st[1] = {P * es};
-    const cuuint32_t box[2] = {bx, (cuuint32_t)Q};
-    ok = ok && encode_map(&m.h, t, 2, d.h_in, dims, st, box);
-  }
-  {
-    const cuuint64_t dims[3] = {P, (cuuint64_t)C, (cuuint64_t)NJ}, st[2] = {P * es, C * P * es};
-    const cuuint32_t box[3] = {bx, 1, (cuuint32_t)NJ};
-    ok = ok && encode_map(&m.f3, t, 3, d.f_in, dims, st, box);
-  }
-  if (Split<L>::nf(0) > NJ) {
-    const cuuint64_t dims[2] = {P, (cuuint64_t)NJ + 1}, st[1] = {C * P * es};
-    const cuuint32_t box[2] = {bx, (cuuint32_t)NJ + 1};
-    ok = ok && encode_map(&m.f4, t, 2, d.f_in, dims, st, box);
-  }
-  {
-    static_assert(sizeof(typename Store<S>::X) == 4, "chi is staged as 4-byte values");
-    const cuuint64_t dims[2] = {P, (cuuint64_t)C}, st[1] = {P * 4};
-    const cuuint32_t box[2] = {bx, 1};
-    ok = ok && encode_map(&m.x, tf, 2, d.chi, dims, st, box);
-  }
+  auto rows = [&](CUtensorMap* mp, CUtensorMapDataType ty, cuuint64_t sz, const void* base, int n) {
+    const cuuint64_t dims[2] = {P, (cuuint64_t)n}, st[1] = {P * sz};
+    const cuuint32_t box[2] = {bx, (cuuint32_t)n};
+    ok = ok && encode_map(mp, ty, 2, base, dims, st, box);
+  };
+  rows(&m.f, t, es, f, Q);
+  rows(&m.x, xs == 8 ? td : tf, xs, chi, C);
   if constexpr (Store<S>::V2) {
-    const char* h0 = static_cast<const char*>(d.h_in) + es * C * Q * P;
-    const char* U = static_cast<const char*>(d.f_in) + es * Q * P;
+    const char* h0 = static_cast<const char*>(h) + es * C * Q * P;
+    const char* U = static_cast<const char*>(f) + es * Q * P;
     if (!aligned(h0) || !aligned(U)) return m;
-    {
-      const cuuint64_t dims[2] = {P, (cuuint64_t)C}, st[1] = {P * 4};
-      const cuuint32_t box[2] = {bx, 1};
-      ok = ok && encode_map(&m.e0, tf, 2, h0, dims, st, box);
-    }
-    {
-      const cuuint64_t dims[2] = {P, (cuuint64_t)D}, st[1] = {P * 4};
-      const cuuint32_t box[2] = {bx, (cuuint32_t)D};
-      ok = ok && encode_map(&m.u, tf, 2, U, dims, st, box);
-    }
+    rows(&m.e0, tf, 4, h0, C);
+    rows(&m.u, tf, 4, U, D);
+    // (the i = 0 slots are unused: directions 1 .. Q - 1 of every component)
+    const cuuint64_t dims[3] = {P, (cuuint64_t)Q, (cuuint64_t)C}, st[2] = {P * es, Q * P * es};
+    const cuuint32_t box[3] = {bx, (cuuint32_t)(Q - 1), (cuuint32_t)C};
+    ok = ok && encode_map(&m.h, t, 3, h, dims, st, box);
+  } else {
+    rows(&m.h, t, es, h, C * Q);
   }
   m.on = ok ? 1 : 0;
   return m;
@@ -178,89 +154,103 @@ cudaError_t allow_dynamic_smem(K* kern, size_t bytes) {
   return e;
 }
 
-// Launch a fused-step kernel instance; a tile of more than 48 KB of shared
-// memory (XN > 1) is given it dynamically.
-template <class L, class S, int GX, int TY, int MINB, bool WALLS, bool FW, bool CL, int XN,
-          bool ORIG = false>
-cudaError_t launch_kernel(dim3 grid, const StepDesc& d, const Grid& g, const Phys<RT<S>>& ph,
-                          const Bufs<S>& b, int mchunk, const StageMaps& tm) {
-  constexpr int NT = FusedShape<L, GX, TY, FW, XN, fill_warps_max<S, XN>()>::NT;
-  constexpr size_t dyn = TileCfg<L, S, GX, TY, FW, CL, XN, MINB>::kDynamicBytes;
-  auto kern = k_step_fused<L, S, GX, TY, MINB, WALLS, FW, CL, XN, ORIG>;
-  if constexpr (dyn > 0) {
-    const cudaError_t e = allow_dynamic_smem(kern, dyn);
-    if (e != cudaSuccess) return e;
+// Tile shapes of the fused step: 32 GX nodes along x, KG threads per node,
+// MINB resident blocks per SM (registers and stage buffers are budgeted for
+// them).  Measured on GB300, MLUPS (the 256^3 / 2048^2 periodic flows; in
+// brackets the kernel with one thread per stress component):
+//   D3Q19 FP32 2,2,2: 5680 (5244); KG 1: 5517, KG 3: 5616, GX 1: 4683
+//   D3Q19 FP16 2,2,3: 6463 (4803); KG 1: 5562, MINB 2: 6188, GX 1: 4961
+//   D3Q19 FP64 (96^3) 1,2,2: 567 (343); KG 1: 371, KG 3: 540, KG 6: 430
+//   D2Q9 FP32 4,1,2: 19180 (18102); KG 3: 18223, GX 2: 19012
+//   D2Q9 FP16 4,1,4: 27500 (14835); MINB 3: 25590, 5: 23250, GX 2: 23520
+//   D2Q9 FP64 (512^2) 2,1,3: 2060 (948); KG 3: 1463, GX 4: 1968
+// SMALL: one warp's nodes per tile, for grids that leave the chip idle
+// otherwise (the larger KG spreads FP64 over the four quarters of an SM).
+template <class L, class S, bool SMALL>
+struct StepShape {
+  static constexpr int B = sizeof(S);
+  static constexpr int GX = L::D == 3 ? (SMALL || B == 8 ? 1 : 2) : (SMALL ? 1 : (B == 8 ? 2 : 4));
+  static constexpr int KG = L::D == 3 ? 2 : (SMALL && B == 8 ? 3 : 1);
+  static constexpr int MINB = L::D == 3 ? (SMALL ? (B == 2 ? 4 : 3) : (B == 2 ? 3 : 2))
+                                        : (SMALL ? (B == 8 ? 3 : 4) : (B == 2 ? 4 : (B == 8 ? 3 : 2)));
+};
+
+// Planes per block along the march axis, for `tiles` tiles of a plane, `nm`
+// planes and `slots` resident blocks.  A block's time is its planes plus the
+// prologue (three planes of the velocity ring and the first copies, about
+// kPrologue planes); the grid takes blocks / slots such times, rounded up
+// while the waves are few.
+inline int pick_chunk(long long tiles, int nm, long long slots, double* cost_out = nullptr) {
+  constexpr double kPrologue = 2.5;
+  constexpr int kMost = 32;
+  const int least = (nm + 65534) / 65535;   // the chunks are the grid's z extent
+  int best = least;
+  double cost = 1e300;
+  for (int c = least; c <= std::max(least, std::min(nm, kMost)); ++c) {
+    const long long blocks = tiles * ((nm + c - 1) / c);
+    double w = (double)blocks / (double)slots;
+    w = w < 4.0 ? std::ceil(w) : w + 0.5;
+    const double t = w * (c + kPrologue);
+    if (t <= cost) {
+      cost = t;
+      best = c;
+    }
   }
-  kern<<<grid, NT, dyn, d.stream>>>(g, ph, b, mchunk, tm);
+  if (cost_out) *cost_out = cost;
+  return best;
+}
+
+template <class L, class S, int GX, int KG, int MINB, bool WALLS, bool PADDED, bool CL, bool ORIG>
+cudaError_t launch_kernel(const StepDesc& d, const Grid& g, const Phys<RT<S>>& ph,
+                          const Bufs<S>& b) {
+  using Sh = FusedShape<L, S, GX, KG>;
+  using Cfg = TileCfg<L, S, GX, KG, MINB, PADDED, CL>;
+  auto kern = k_step_fused<L, S, GX, KG, MINB, WALLS, PADDED, CL, ORIG>;
+  const cudaError_t e = allow_dynamic_smem(kern, sizeof(typename Cfg::Smem));
+  if (e != cudaSuccess) return e;
+  const int bx = (d.nx + Sh::TXS - 1) / Sh::TXS;
+  const int by = L::D == 3 ? d.ny : 1;
+  const int nm = L::D == 3 ? g.nz : d.ny;
+  const int mchunk = pick_chunk((long long)bx * by, nm, (long long)std::max(d.sms, 1) * MINB);
+  const StageMaps tm = stage_maps<L, S>(b.f_in, b.h_in, b.chi, d.pitch, Cfg::BX);
+  kern<<<dim3(bx, by, (nm + mchunk - 1) / mchunk), Sh::NT, sizeof(typename Cfg::Smem), d.stream>>>(
+      g, ph, b, mchunk, tm);
   return cudaGetLastError();
 }
 
-template <class L, class S, int GX, int TY, int MINB, bool FW, int XN = 1, bool ORIG = false>
+// The kernel variant of a grid: row starts on 16-byte boundaries need no
+// padded stage; padded tiles serve walled and periodic grids alike.
+template <class L, class S, int GX, int KG, int MINB, bool CL, bool ORIG>
 cudaError_t launch_fused(const StepDesc& d, const Grid& g, const Phys<RT<S>>& ph,
                          const Bufs<S>& b) {
-  constexpr int TXS = GX * 32 * XN;
-  const int bx = (d.nx + TXS - 1) / TXS;
-  const int by = L::D == 3 ? (d.ny + TY - 1) / TY : 1;
-  const int nm = L::D == 3 ? g.nz : d.ny;
-  // chunks along the march axis: enough blocks for several waves, but at
-  // least `min_chunk` planes so the two halo planes stay a small overhead
-  const int waves = tune_int("FVLB_WAVES", L::D == 2 ? 4 : 16);
-  const int min_chunk = tune_int("FVLB_MIN_CHUNK", 8);
-  const long long target = (long long)std::max(d.sms, 1) * MINB * waves;
-  int nchunk = (int)std::max<long long>(1, target / std::max(1, bx * by));
-  int mchunk = std::max(min_chunk, (nm + nchunk - 1) / nchunk);
-  mchunk = std::min(mchunk, nm);
-  nchunk = (nm + mchunk - 1) / mchunk;
-  dim3 grid(bx, by, nchunk);
-  StageMaps tm;
-  std::memset(&tm, 0, sizeof tm);
-  if constexpr (TileCfg<L, S, GX, TY, FW, false, XN, MINB>::PF) tm = stage_maps<L, S>(d, 32 * XN);
-  if constexpr (std::is_same<S, float>::value && XN == 1 && !ORIG && (L::D == 3 || !FW)) {
-    if (d.mlp) {  // learned closure (FP32 storage only); two blocks per SM
-      if (d.walls) return launch_kernel<L, S, GX, TY, 2, true, FW, true, 1>(grid, d, g, ph, b, mchunk, tm);
-      return launch_kernel<L, S, GX, TY, 2, false, FW, true, 1>(grid, d, g, ph, b, mchunk, tm);
-    }
-  }
-  if (d.walls)
-    return launch_kernel<L, S, GX, TY, MINB, true, FW, false, XN, ORIG>(grid, d, g, ph, b, mchunk, tm);
-  return launch_kernel<L, S, GX, TY, MINB, false, FW, false, XN, ORIG>(grid, d, g, ph, b, mchunk, tm);
+  if (d.nx % (16 / (int)sizeof(S)))
+    return launch_kernel<L, S, GX, KG, MINB, true, true, CL, ORIG>(d, g, ph, b);
+  if (d.walls) return launch_kernel<L, S, GX, KG, MINB, true, false, CL, ORIG>(d, g, ph, b);
+  return launch_kernel<L, S, GX, KG, MINB, false, false, CL, ORIG>(d, g, ph, b);
 }
 
-// The fused step in the shape measured fastest on GB300 (256^3 D3Q19, 2048^2
-// D2Q9): 2D four 32-node groups x 3 components + 5 (FP32) or 4 (16-bit) halo
-// fill warps (544 / 512 threads, 2 blocks per SM; FP64 and the learned
-// closure without fill warps, 384 threads); 3D FP32 and 16-bit a 64-node row, each of the 6 component warps
-// taking its two 32-node halves in turn, + 7 (FP32) or 4 (16-bit) halo fill
-// warps (416 / 320 threads, 2 blocks per SM; a 64-register cap for 3 blocks
-// per SM measured slower); 3D FP64 and the learned closure one 32-node row
-// with 4 fill warps.  ORIG: the original scheme's
-// step (div tau_p from ph.fdiv in the body force, f^B off).
+// The fused step.  ORIG: the original scheme's step (div tau_p from ph.fdiv in
+// the body force, f^B off).
 template <class L, class S, bool ORIG>
 cudaError_t fused_step(const StepDesc& d, const Grid& g, const Phys<RT<S>>& ph,
                        const Bufs<S>& b) {
-  constexpr bool wide = sizeof(RT<S>) == 8;
-  if constexpr (L::D == 2) {
-    // 4 groups x 3 components; FP64 and the learned closure fill the ring
-    // in the collision threads, FP32 and 16-bit storage with fill warps
-    if constexpr (wide) {
-      return launch_fused<L, S, 4, 1, 1, false, 1, ORIG>(d, g, ph, b);
-    } else {
-      if constexpr (!ORIG) {
-        if (d.mlp) return launch_fused<L, S, 4, 1, 2, false, 1>(d, g, ph, b);
-      }
-      return launch_fused<L, S, 4, 1, 2, true, 1, ORIG>(d, g, ph, b);
-    }
-  } else {
-    if constexpr (wide) return launch_fused<L, S, 1, 1, 1, true, 1, ORIG>(d, g, ph, b);
-    else if constexpr (sizeof(S) == 4) {
-      if constexpr (!ORIG) {
-        if (d.mlp) return launch_fused<L, S, 1, 1, 2, true, 1>(d, g, ph, b);
-      }
-      return launch_fused<L, S, 1, 1, 2, true, 2, ORIG>(d, g, ph, b);
-    } else {
-      return launch_fused<L, S, 1, 1, 2, true, 2, ORIG>(d, g, ph, b);
-    }
+  using Big = StepShape<L, S, false>;
+  using Small = StepShape<L, S, true>;
+  if constexpr (std::is_same<S, float>::value && !ORIG) {
+    if (d.mlp) return launch_fused<L, S, Big::GX, (L::D == 3 ? 2 : 1), 2, true, false>(d, g, ph, b);
   }
+  if constexpr (Big::GX != Small::GX) {
+    const int by = L::D == 3 ? d.ny : 1, nm = L::D == 3 ? g.nz : d.ny;
+    auto cost = [&](int gx, int minb) {
+      double c;
+      pick_chunk((long long)((d.nx + 32 * gx - 1) / (32 * gx)) * by, nm,
+                 (long long)std::max(d.sms, 1) * minb, &c);
+      return c;
+    };
+    if (cost(Small::GX, Small::MINB) < cost(Big::GX, Big::MINB))
+      return launch_fused<L, S, Small::GX, Small::KG, Small::MINB, false, ORIG>(d, g, ph, b);
+  }
+  return launch_fused<L, S, Big::GX, Big::KG, Big::MINB, false, ORIG>(d, g, ph, b);
 }
 
 template <class L, class S>
