@@ -71,6 +71,7 @@ struct fvlb_s {
   fvlb_mlp_t mlp = nullptr; // learned closure, or null
   double cl_tol = 1e-2;
   unsigned long long* cl_count = nullptr;  // [0] network nodes, [1] fallbacks
+  fvlb::StepPlan plan;      // of the fused step's launcher
   unsigned* dev_err = nullptr;  // bounded device waits that ran out (bit 0: staging copies)
   int scheme = FVLB_SCHEME_PRESENT;
   void* taup = nullptr;     // original scheme: polymer stress working array
@@ -142,6 +143,7 @@ void free_all(fvlb_t h) {
   h->dev_err = nullptr;
   h->taup = nullptr;
   h->fdiv = nullptr;
+  h->plan = fvlb::StepPlan();
   h->allocated = false;
 }
 
@@ -181,6 +183,8 @@ StepDesc make_desc(fvlb_t h) {
   d.model = h->model;
   d.mpar = h->mpar;
   d.err = h->dev_err;
+  d.plan = &h->plan;
+  d.parity = h->cur;
   double c = 0.0;
   if (h->force.kind == FVLB_FORCE_CONST) c = 1.0;
   if (h->force.kind == FVLB_FORCE_COSINE) c = std::cos(h->force.omega * (double)h->t);

@@ -1076,10 +1076,17 @@ __global__ void __launch_bounds__(FusedShape<L, S, GX, KG>::NT, MINB)
   extern __shared__ __align__(128) unsigned char fvlb_tile_smem[];
   auto& sm = *reinterpret_cast<typename Cfg::Smem*>(fvlb_tile_smem);
   if (threadIdx.x == FusedShape<L, S, GX, KG>::NCW * 32) stage_barriers_init(sm.bar);
+  pdl_wait();   // nothing above reads or writes global memory
   if constexpr (CL) mlp_load(sm.cls.P, static_cast<const MlpPacked*>(ph.mlp));
   StagePos pos;
   fused_tile<L, S, GX, KG, MINB, WALLS, PADDED, CL, ORIG>(sm, g, ph, b, mchunk, blockIdx.x,
                                                       blockIdx.y, blockIdx.z, &tm, tm.on != 0, pos);
+  // The next step's blocks may come in when every block's first collision warp
+  // is through.  (Earlier, they take the free slots of SMs that are busy with
+  // this step: 64^2 FP64 17.3 us a step with the trigger at the start, 11.1
+  // at the last plane, 11.0 here, 12.3 without; 128^2 FP32 3.75, 3.67, 3.12
+  // and 6.15; 517 x 333 FP32 11.2, 11.0, 10.8 and 12.5; large grids the same.)
+  if (threadIdx.x < FusedShape<L, S, GX, KG>::NCW * 32) pdl_trigger();
 }
 
 // ---------------------------------------------------------------------------

@@ -29,6 +29,19 @@ inline double bytes_per_update(int storage, int Q, int C, int D) {
   return 2.0 * (Q * sb + 4.0 * D + C * (Q - 1) * sb + 4.0 * C) + 2.0 * C * xb;
 }
 
+// What the fused step's launcher works out once per handle: the kernel
+// instance it was worked out for, its planes per block, the choice of the
+// one-warp tile (-1: not made), and the tensor maps of the two parities
+// (StageMaps; -1: not encoded).  A handle's grid and buffers do not change
+// after allocation.
+struct StepPlan {
+  const void* kern = nullptr;
+  int mchunk = 0;
+  int small = -1;
+  int mapped[2] = {-1, -1};
+  alignas(128) unsigned char maps[2][768];
+};
+
 // Precision-agnostic description of one launch; the launcher converts the
 // physics to the working precision of the storage type.
 struct StepDesc {
@@ -59,6 +72,8 @@ struct StepDesc {
   void* fdiv;           // original scheme, fused variant: D * pitch working-precision values
   int model;            // constitutive model (0 Oldroyd-B, 1 Giesekus, 2 / 3 PTT)
   double mpar;          // its parameter
+  StepPlan* plan;       // the handle's plan, or null
+  int parity;           // which of the handle's buffers f_in / h_in are
   unsigned* err;        // device word: bounded waits that ran out (bit 0: staging copies)
 };
 

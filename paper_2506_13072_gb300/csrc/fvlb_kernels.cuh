@@ -98,6 +98,12 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
+// Programmatic dependent launch: let the next kernel of the stream start its
+// blocks while this one drains, and wait until the previous one has finished
+// and its writes are visible.  Without a programmatic edge both do nothing.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
 // Tensor maps of one launch's staged arrays (the fused step's copies of a
 // tile's row of nodes into its stage), encoded on the host; `on` = 0: the
 // lanes copy their own nodes instead.  Dimension 0 is the node index within

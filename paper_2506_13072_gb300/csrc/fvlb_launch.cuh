@@ -200,22 +200,50 @@ inline int pick_chunk(long long tiles, int nm, long long slots, double* cost_out
   return best;
 }
 
+// Launch with a programmatic edge to the previous kernel of the stream: the
+// blocks may start while it drains, and wait for its end themselves (pdl_wait).
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream,
+                       const A&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 template <class L, class S, int GX, int KG, int MINB, bool WALLS, bool PADDED, bool CL, bool ORIG>
 cudaError_t launch_kernel(const StepDesc& d, const Grid& g, const Phys<RT<S>>& ph,
                           const Bufs<S>& b) {
   using Sh = FusedShape<L, S, GX, KG>;
   using Cfg = TileCfg<L, S, GX, KG, MINB, PADDED, CL>;
   auto kern = k_step_fused<L, S, GX, KG, MINB, WALLS, PADDED, CL, ORIG>;
-  const cudaError_t e = allow_dynamic_smem(kern, sizeof(typename Cfg::Smem));
-  if (e != cudaSuccess) return e;
   const int bx = (d.nx + Sh::TXS - 1) / Sh::TXS;
   const int by = L::D == 3 ? d.ny : 1;
   const int nm = L::D == 3 ? g.nz : d.ny;
-  const int mchunk = pick_chunk((long long)bx * by, nm, (long long)std::max(d.sms, 1) * MINB);
-  const StageMaps tm = stage_maps<L, S>(b.f_in, b.h_in, b.chi, d.pitch, Cfg::BX);
-  kern<<<dim3(bx, by, (nm + mchunk - 1) / mchunk), Sh::NT, sizeof(typename Cfg::Smem), d.stream>>>(
-      g, ph, b, mchunk, tm);
-  return cudaGetLastError();
+  static_assert(sizeof(StageMaps) <= sizeof(StepPlan::maps[0]), "room for the tensor maps");
+  StepPlan once;
+  StepPlan& pl = d.plan ? *d.plan : once;
+  if (pl.kern != reinterpret_cast<const void*>(kern)) {
+    const cudaError_t e = allow_dynamic_smem(kern, sizeof(typename Cfg::Smem));
+    if (e != cudaSuccess) return e;
+    pl.mchunk = pick_chunk((long long)bx * by, nm, (long long)std::max(d.sms, 1) * MINB);
+    pl.mapped[0] = pl.mapped[1] = -1;
+    pl.kern = reinterpret_cast<const void*>(kern);
+  }
+  StageMaps& tm = *reinterpret_cast<StageMaps*>(pl.maps[d.parity & 1]);
+  if (pl.mapped[d.parity & 1] < 0) {
+    tm = stage_maps<L, S>(b.f_in, b.h_in, b.chi, d.pitch, Cfg::BX);
+    pl.mapped[d.parity & 1] = tm.on;
+  }
+  return launch_pdl(kern, dim3(bx, by, (nm + pl.mchunk - 1) / pl.mchunk), Sh::NT,
+                    sizeof(typename Cfg::Smem), d.stream, g, ph, b, pl.mchunk, tm);
 }
 
 // The kernel variant of a grid: row starts on 16-byte boundaries need no
@@ -247,7 +275,12 @@ cudaError_t fused_step(const StepDesc& d, const Grid& g, const Phys<RT<S>>& ph,
                  (long long)std::max(d.sms, 1) * minb, &c);
       return c;
     };
-    if (cost(Small::GX, Small::MINB) < cost(Big::GX, Big::MINB))
+    int small = d.plan ? d.plan->small : -1;
+    if (small < 0) {
+      small = cost(Small::GX, Small::MINB) < cost(Big::GX, Big::MINB);
+      if (d.plan) d.plan->small = small;
+    }
+    if (small)
       return launch_fused<L, S, Small::GX, Small::KG, Small::MINB, false, ORIG>(d, g, ph, b);
   }
   return launch_fused<L, S, Big::GX, Big::KG, Big::MINB, false, ORIG>(d, g, ph, b);
