@@ -188,99 +188,171 @@ __device__ __forceinline__ void fused_tile(
   const int warp = tid >> 5, lane = tid & 31;
   auto slot = [&](int q) { return (q - m0 + 1) & 3; };
   auto plane_of = [&](int q) -> int {  // -1: beyond a wall
-    if (q < 0 || q >= nm) return wall_m ? -1 : (q + nm) % nm;
+    // (planes -1 .. nm are used: one wrap at most)
+    if (q < 0) return wall_m ? -1 : q + nm;
+    if (q >= nm) return wall_m ? -1 : q - nm;
     return q;
+  };
+  // ring slot (ex, ey)'s node, one node outside the tile on each side: none
+  // beyond a wall, and none past the slot after the row's last node
+  auto ring_node = [&](int ex, int ey, int& gx, int& gy) -> bool {
+    gx = x0 + ex - 1;
+    gy = (D == 3) ? y + ey - 1 : 0;
+    bool has = gx <= nx;
+    if (gx < 0 || gx == nx) {
+      if (wall_x) has = false;
+      gx = gx < 0 ? nx - 1 : 0;
+    }
+    if (D == 3 && (gy < 0 || gy == ny)) {
+      if (wall_y) has = false;
+      gy = gy < 0 ? ny - 1 : 0;
+    }
+    return has;
   };
   auto node_of = [&](int mm, int gx, int gy) -> uint32_t {
     return (D == 3) ? ((uint32_t)mm * (uint32_t)ny + (uint32_t)gy) * (uint32_t)nx + (uint32_t)gx
                     : (uint32_t)mm * (uint32_t)nx + (uint32_t)gx;
   };
 
+  // Velocity of ring slot e of plane q from its momentum sums `mo` (when
+  // `ok`), into the ring.
+  auto ring_store = [&](int e, bool ok, int mm, int gx, int gy, const R (&mo)[D],
+                        const R (&Ub)[D], int q) {
+    R u[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) u[a] = R(0);
+    if (ok) {
+      R F[3];
+      body_force<L, R>(ph, gx, D == 3 ? gy : mm, F);
+      if constexpr (ORIG) {  // the original scheme: + div tau_p of this node
+        const uint32_t sf = node_of(mm, gx, gy);
+#pragma unroll
+        for (int a = 0; a < D; ++a) F[a] += ph.fdiv[(uint32_t)a * P32 + sf];
+      }
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        // 16-bit forms: u = U + sum_i c_i s_i / KF + F/2 (the velocity part
+        // e_i(U) of the stored deviations carries momentum U and no other
+        // first moment)
+        if constexpr (V2) u[a] = mo[a] * R(1.0f / Store<S>::KF) + Ub[a] + R(0.5) * F[a];
+        else u[a] = mo[a] + R(0.5) * F[a];
+      }
+    }
+    Vel<R, D> t;
+#pragma unroll
+    for (int a = 0; a < D; ++a) t.v[a] = u[a];
+    if constexpr (D == 3) t.v[3] = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];  // |u|^2
+    ring[slot(q)][e] = t;
+  };
+  // the same from raw 16-bit populations: each enters the momentum sums
+  // with one mixed-precision add or subtract, the accumulator's sign
+  // tracked at compile time (f - v = -(v - f) exactly)
+  auto bits_store = [&](int e, bool ok, int mm, int gx, int gy, const unsigned short (&sb)[Q],
+                        const R (&Ub)[D], int q) {
+    if constexpr (V2) {
+      R mo[D];
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        R v = R(0);
+        bool neg = false;   // v = -(momentum sum) while set
+#pragma unroll
+        for (int i = 1; i < Q; ++i) {
+          const int c = cc<L>(i, a);
+          if (c == 0) continue;
+          if ((c == 1) != neg) {
+            v = Store<S>::accb(v, sb[i]);
+          } else {
+            v = Store<S>::subb(sb[i], v);
+            neg = !neg;
+          }
+        }
+        mo[a] = neg ? -v : v;
+      }
+      ring_store(e, ok, mm, gx, gy, mo, Ub, q);
+    }
+  };
+
+  // one ring slot's populations: loaded, then turned into its velocity
+  struct Held {
+    S f[Q];
+    R u[D];
+  };
+  auto slot_load = [&](bool has, int mm, int gx, int gy, Held& v) {
+    if (has && mm >= 0) {
+      const uint32_t s = node_of(mm, gx, gy);
+#pragma unroll
+      for (int i = 1; i < Q; ++i) v.f[i] = b.f_in[(uint32_t)i * P32 + s];
+      if constexpr (V2) {
+        const float* U = f_ext<L>(b.f_in, P);
+#pragma unroll
+        for (int a = 0; a < D; ++a) v.u[a] = __ldg(U + ((uint32_t)a * P32 + s));
+      }
+    }
+  };
+  auto slot_store = [&](int e, bool has, int mm, int gx, int gy, int q, const Held& v) {
+    const bool ok = has && mm >= 0;
+    if constexpr (V2) {
+      unsigned short hb[Q];
+      hb[0] = 0;
+#pragma unroll
+      for (int i = 1; i < Q; ++i) hb[i] = *reinterpret_cast<const unsigned short*>(&v.f[i]);
+      bits_store(e, ok, mm, gx, gy, hb, v.u, q);
+    } else {
+      R mo[D];
+      momentum<L, R>(v.f, mo);
+      ring_store(e, ok, mm, gx, gy, mo, mo, q);
+    }
+  };
+  // The first three planes of the ring, by all warps, their loads in flight
+  // together (a chunk of one plane spends more on them than on its own plane).
+  auto prologue = [&]() {
+    constexpr int NPRO = (3 * NE + Sh::NT - 1) / Sh::NT;
+    Held v[NPRO];
+    int gx[NPRO], gy[NPRO], mm[NPRO];
+    bool has[NPRO];
+#pragma unroll
+    for (int t = 0; t < NPRO; ++t) {
+      const int n = tid + t * Sh::NT;
+      const int e = n % NE, pq = n / NE;
+      has[t] = ring_node(e % EX, e / EX, gx[t], gy[t]) && n < 3 * NE;
+      mm[t] = plane_of(m0 - 1 + pq);
+      slot_load(has[t], mm[t], gx[t], gy[t], v[t]);
+    }
+#pragma unroll
+    for (int t = 0; t < NPRO; ++t) {
+      const int n = tid + t * Sh::NT;
+      if (n < 3 * NE) slot_store(n % NE, has[t], mm[t], gx[t], gy[t], m0 - 1 + n / NE, v[t]);
+    }
+  };
+
+  // The first fill thread issues the stage copies of the block.
+  StagePos pst = pos;
+  if (FENCE_MAPS && tma && tid == NCW * 32) fence_tensor_maps(tm);
+  auto produce = [&](int q) {
+    if (!tma || tid != NCW * 32 || q >= m1) return;
+    auto& W = sm.stage[pst.st];
+    uint64_t* bar = &sm.bar[pst.st];
+    pst.template next<NST>();
+    int s0 = (int)node_of(q, x0, y);
+    if constexpr (PADDED) s0 &= ~(Cfg::EPC - 1);
+    fence_proxy_async();   // the collision warps' reads of this buffer (ordered by A) first
+    mbar_arrive_expect_tx(bar, Cfg::kBytes);
+    tma_load_2d(&W.f[0][0], &tm->f, s0, 0, bar);
+    if constexpr (V2) {
+      tma_load_2d(&W.U[0][0], &tm->u, s0, 0, bar);
+      tma_load_2d(&W.h0[0][0], &tm->e0, s0, 0, bar);
+      tma_load_3d(&W.h[0][0][0], &tm->h, s0, 1, 0, bar);
+    } else {
+      tma_load_2d(&W.h[0][0][0], &tm->h, s0, 0, bar);
+    }
+    tma_load_2d(&W.chi[0][0], &tm->x, s0, 0, bar);
+  };
+  produce(m0);
+  if (NST > 2) produce(m0 + 1);
+  prologue();
+
   if (warp >= NCW) {
     // ---------------- fill warps ---------------------------------------------
-    // The first fill thread issues the stage copies of the block.
-    StagePos pst = pos;
-    if (FENCE_MAPS && tma && tid == NCW * 32) fence_tensor_maps(tm);
-    auto produce = [&](int q) {
-      if (!tma || tid != NCW * 32 || q >= m1) return;
-      auto& W = sm.stage[pst.st];
-      uint64_t* bar = &sm.bar[pst.st];
-      pst.template next<NST>();
-      int s0 = (int)node_of(q, x0, y);
-      if constexpr (PADDED) s0 &= ~(Cfg::EPC - 1);
-      fence_proxy_async();   // the collision warps' reads of this buffer (ordered by A) first
-      mbar_arrive_expect_tx(bar, Cfg::kBytes);
-      tma_load_2d(&W.f[0][0], &tm->f, s0, 0, bar);
-      if constexpr (V2) {
-        tma_load_2d(&W.U[0][0], &tm->u, s0, 0, bar);
-        tma_load_2d(&W.h0[0][0], &tm->e0, s0, 0, bar);
-        tma_load_3d(&W.h[0][0][0], &tm->h, s0, 1, 0, bar);
-      } else {
-        tma_load_2d(&W.h[0][0][0], &tm->h, s0, 0, bar);
-      }
-      tma_load_2d(&W.chi[0][0], &tm->x, s0, 0, bar);
-    };
-    produce(m0);
-    if (NST > 2) produce(m0 + 1);
-
-    // Velocity of ring slot e of plane q from its momentum sums `mo` (when
-    // `ok`), into the ring.
-    auto ring_store = [&](int e, bool ok, int mm, int gx, int gy, const R (&mo)[D],
-                          const R (&Ub)[D], int q) {
-      R u[D];
-#pragma unroll
-      for (int a = 0; a < D; ++a) u[a] = R(0);
-      if (ok) {
-        R F[3];
-        body_force<L, R>(ph, gx, D == 3 ? gy : mm, F);
-        if constexpr (ORIG) {  // the original scheme: + div tau_p of this node
-          const uint32_t sf = node_of(mm, gx, gy);
-#pragma unroll
-          for (int a = 0; a < D; ++a) F[a] += ph.fdiv[(uint32_t)a * P32 + sf];
-        }
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-          // 16-bit forms: u = U + sum_i c_i s_i / KF + F/2 (the velocity part
-          // e_i(U) of the stored deviations carries momentum U and no other
-          // first moment)
-          if constexpr (V2) u[a] = mo[a] * R(1.0f / Store<S>::KF) + Ub[a] + R(0.5) * F[a];
-          else u[a] = mo[a] + R(0.5) * F[a];
-        }
-      }
-      Vel<R, D> t;
-#pragma unroll
-      for (int a = 0; a < D; ++a) t.v[a] = u[a];
-      if constexpr (D == 3) t.v[3] = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];  // |u|^2
-      ring[slot(q)][e] = t;
-    };
-    // the same from raw 16-bit populations: each enters the momentum sums
-    // with one mixed-precision add or subtract, the accumulator's sign
-    // tracked at compile time (f - v = -(v - f) exactly)
-    auto bits_store = [&](int e, bool ok, int mm, int gx, int gy, const unsigned short (&sb)[Q],
-                          const R (&Ub)[D], int q) {
-      if constexpr (V2) {
-        R mo[D];
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-          R v = R(0);
-          bool neg = false;   // v = -(momentum sum) while set
-#pragma unroll
-          for (int i = 1; i < Q; ++i) {
-            const int c = cc<L>(i, a);
-            if (c == 0) continue;
-            if ((c == 1) != neg) {
-              v = Store<S>::accb(v, sb[i]);
-            } else {
-              v = Store<S>::subb(sb[i], v);
-              neg = !neg;
-            }
-          }
-          mo[a] = neg ? -v : v;
-        }
-        ring_store(e, ok, mm, gx, gy, mo, Ub, q);
-      }
-    };
-
     if constexpr (Sh::PAIRS) {
       // Even nx and no walls across x: thread pp takes the node pair (x even,
       // x + 1) px of ring row ey, ring slots 2 px - 1 and 2 px (those in the
@@ -289,21 +361,19 @@ __device__ __forceinline__ void fused_tile(
         const int pp = tid - NCW * 32;
         const int ey = pp / Sh::PX, px = pp - ey * Sh::PX;
         const bool pact = pp < Sh::NPR;
-        int gx0 = x0 + 2 * px - 2;                  // even
-        gx0 = ((gx0 % nx) + nx) % nx;               // periodic in x (nx even: stays even)
-        int gy = (D == 3) ? y + ey - 1 : 0;
-        bool has = pact;
-        if (D == 3 && (gy < 0 || gy >= ny)) {
-          if (wall_y) has = false;
-          gy = ((gy % ny) + ny) % ny;
-        }
+        int gx0 = x0 + 2 * px - 2, gy;              // even
+        bool has = pact && gx0 <= nx;
+        if (gx0 < 0) gx0 += nx;                     // periodic in x (nx even: stays even)
+        if (gx0 == nx) gx0 = 0;
+        int gxn;
+        has = ring_node(1, ey, gxn, gy) && has;     // (the row's gy)
         const int ea = ey * EX + 2 * px - 1;        // slot of node gx0 (px > 0)
         const bool sa = pact && px > 0, sb = pact && 2 * px < EX;
-        struct Held {
+        struct Pair {
           uint32_t f[Q];
           float2 u[D];
         };
-        auto pload = [&](int mm, Held& v) {
+        auto pload = [&](int mm, Pair& v) {
           if (has && mm >= 0) {
             const uint32_t s0 = node_of(mm, gx0, gy);
             const uint32_t* fw = reinterpret_cast<const uint32_t*>(b.f_in);
@@ -315,7 +385,7 @@ __device__ __forceinline__ void fused_tile(
               v.u[a] = __ldg(reinterpret_cast<const float2*>(U + ((uint32_t)a * P32 + s0)));
           }
         };
-        auto pstore = [&](int mm, int q, const Held& v) {
+        auto pstore = [&](int mm, int q, const Pair& v) {
           const bool ok = has && mm >= 0;
 #pragma unroll
           for (int n = 0; n < 2; ++n) {
@@ -330,18 +400,7 @@ __device__ __forceinline__ void fused_tile(
             bits_store(ea + n, ok, mm, gx0 + n, gy, hb, Ub, q);
           }
         };
-        Held v;
-        {
-          // the first two planes' loads in flight together
-          Held v1;
-          const int q0 = plane_of(m0 - 1), q1 = plane_of(m0), q2 = plane_of(m0 + 1);
-          pload(q0, v);
-          pload(q1, v1);
-          pstore(q0, m0 - 1, v);
-          pload(q2, v);
-          pstore(q1, m0, v1);
-          pstore(q2, m0 + 1, v);
-        }
+        Pair v;
         int mq = plane_of(m0 + 2);
         if (m0 + 2 <= m1) pload(mq, v);
         for (int m = m0; m < m1; ++m) {
@@ -365,74 +424,14 @@ __device__ __forceinline__ void fused_tile(
 #pragma unroll
     for (int t = 0; t < SPF; ++t) {
       const int e = e0 + t * NFW * 32;
-      const int ex = e % EX, ey = e / EX;
-      bool has = e < NE;
-      int gx = x0 + ex - 1, gy = (D == 3) ? y + ey - 1 : 0;
-      if (gx < 0 || gx >= nx) {
-        if (wall_x) has = false;
-        gx = ((gx % nx) + nx) % nx;
-      }
-      if (D == 3 && (gy < 0 || gy >= ny)) {
-        if (wall_y) has = false;
-        gy = ((gy % ny) + ny) % ny;
-      }
-      sgx[t] = gx;
-      sgy[t] = gy;
-      shas[t] = has;
+      shas[t] = ring_node(e % EX, e / EX, sgx[t], sgy[t]) && e < NE;
     }
-    struct Held {
-      S f[Q];
-      R u[D];
-    };
-    auto fload = [&](int t, int mm, Held& v) {
-      if (shas[t] && mm >= 0) {
-        const uint32_t s = node_of(mm, sgx[t], sgy[t]);
-#pragma unroll
-        for (int i = 1; i < Q; ++i) v.f[i] = b.f_in[(uint32_t)i * P32 + s];
-        if constexpr (V2) {
-          const float* U = f_ext<L>(b.f_in, P);
-#pragma unroll
-          for (int a = 0; a < D; ++a) v.u[a] = __ldg(U + ((uint32_t)a * P32 + s));
-        }
-      }
-    };
+    auto fload = [&](int t, int mm, Held& v) { slot_load(shas[t], mm, sgx[t], sgy[t], v); };
     auto fstore = [&](int t, int mm, int q, const Held& v) {
       const int e = e0 + t * NFW * 32;
-      if (e >= NE) return;
-      const bool ok = shas[t] && mm >= 0;
-      R mo[D];
-      if constexpr (V2) {
-        unsigned short hb[Q];
-        hb[0] = 0;
-#pragma unroll
-        for (int i = 1; i < Q; ++i) hb[i] = *reinterpret_cast<const unsigned short*>(&v.f[i]);
-        bits_store(e, ok, mm, sgx[t], sgy[t], hb, v.u, q);
-      } else {
-        momentum<L, R>(v.f, mo);
-        ring_store(e, ok, mm, sgx[t], sgy[t], mo, mo, q);
-      }
+      if (e < NE) slot_store(e, shas[t], mm, sgx[t], sgy[t], q, v);
     };
     Held v[SPF];
-    if constexpr (SPF == 1 && !F64) {
-      // the first two planes' loads in flight together
-      Held v1;
-      const int q0 = plane_of(m0 - 1), q1 = plane_of(m0), q2 = plane_of(m0 + 1);
-      fload(0, q0, v[0]);
-      fload(0, q1, v1);
-      fstore(0, q0, m0 - 1, v[0]);
-      fload(0, q2, v[0]);
-      fstore(0, q1, m0, v1);
-      fstore(0, q2, m0 + 1, v[0]);
-    } else {
-#pragma unroll 1
-      for (int q = m0 - 1; q <= m0 + 1; ++q) {
-        const int mm = plane_of(q);
-#pragma unroll
-        for (int t = 0; t < SPF; ++t) fload(t, mm, v[t]);
-#pragma unroll
-        for (int t = 0; t < SPF; ++t) fstore(t, mm, q, v[t]);
-      }
-    }
     int mq = plane_of(m0 + 2);
     if (m0 + 2 <= m1) {
 #pragma unroll
