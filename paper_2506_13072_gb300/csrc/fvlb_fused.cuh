@@ -241,7 +241,10 @@ __device__ __forceinline__ void fused_tile(
     Vel<R, D> t;
 #pragma unroll
     for (int a = 0; a < D; ++a) t.v[a] = u[a];
-    if constexpr (D == 3) t.v[3] = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];  // |u|^2
+    if constexpr (D == 3) {  // |u|^2
+        if constexpr (F64) t.v[3] = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+        else t.v[3] = __fmaf_rn(u[2], u[2], __fmaf_rn(u[0], u[0], __fmul_rn(u[1], u[1])));
+      }
     ring[slot(q)][e] = t;
   };
   // the same from raw 16-bit populations: each enters the momentum sums
@@ -478,12 +481,13 @@ __device__ __forceinline__ void fused_tile(
     __syncwarp();
     asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(KG * 32) : "memory");
   };
-  // FP32 storage fixes the order and the fused multiply-adds of the collision
-  // that its long-run accuracy was established with, whatever the compiler
-  // would contract (another rounding of a slow flow's pressure differs by as
-  // much as its error); FP64 and the 16-bit forms share more between
-  // directions and leave the contraction to the compiler
-  constexpr bool ORD = RS;
+  // FP32 arithmetic fixes the order and the fused multiply-adds of the
+  // collision that its long-run accuracy was established with, whatever the
+  // compiler would contract: another rounding of a slow flow's pressure
+  // differs by as much as its error, and with 16-bit storage one flipped
+  // rounding changes all later ones.  FP64 shares more between directions and
+  // leaves the contraction to the compiler.
+  constexpr bool ORD = !F64;
 
   const R om = ph.inv_tau_h;
   const R keep = R(1) - om;
@@ -740,6 +744,7 @@ __device__ __forceinline__ void fused_tile(
     R bax[KC], bdg[ORD ? KC : 1];       // w_i beta (not ORD: beta)
     R alf[ORD && D == 2 ? KC : 1];      // alpha
     R rest[KC];                         // towards the rest population
+    R h0p[V2 ? KC : 1];                 // 16-bit forms: it, before the rounding residuals
     constexpr double kWx = weight_sum_excess<L, R>();
 #pragma unroll
     for (int q = 0; q < KC; ++q) {
@@ -774,7 +779,9 @@ __device__ __forceinline__ void fused_tile(
         rest[q] = R(0);
         own[q] += src;                             // the zeroth moment, for the end
       } else if constexpr (V2) {
-        rest[q] = (keep * W.h0[k][col] + R(L::w(0)) * alpha) - R(kWx) * alpha;
+        rest[q] = R(0);
+        h0p[q] = __fmaf_rn(-R(kWx), alpha,
+                           __fmaf_rn(keep, W.h0[k][col], __fmul_rn(R(L::w(0)), alpha)));
       } else {
         rest[q] = keep * Store<S>::cvt(Wh[k][0][col]) + R(L::w(0)) * alpha;
       }
@@ -800,7 +807,7 @@ __device__ __forceinline__ void fused_tile(
         Us[a] = W.U[a][col];
         UU += Us[a] * Us[a];
       }
-      sumf += R(1.5 * L::w(0)) * UU;
+      sumf = __fmaf_rn(R(1.5 * L::w(0)), UU, sumf);
     }
     const R kB = ORIG ? R(0) : ph.eta_over_lam * ph.inv_tau_f;
     FBTerms<L, R> fb = {};
@@ -822,10 +829,13 @@ __device__ __forceinline__ void fused_tile(
     for (int a = 0; a < D; ++a) Fd[a] = F64 ? kf * F[a] : F[a];
     const R kFu = kf * Fu;
 
-    uint32_t rng = Store<S>::sr
-                       ? hash32((s * 8u + (uint32_t)kg) * 0x9e3779b9u ^ hash32(ph.step))
-                       : 0u;
-    auto rnd = [&]() -> uint32_t { return Store<S>::sr ? lcg_next(rng) : 0u; };
+    // stochastic rounding: one stream per node and component k, whose draw i is
+    // for h_{k,i} and draw Q + j for f_{k + j C}
+    const uint32_t hs = Store<S>::sr ? hash32(ph.step) : 0u;
+    auto rnd = [&](int k, int n) -> uint32_t {
+      return Store<S>::sr ? lcg_at(hash32((s * 8u + (uint32_t)k) * 0x9e3779b9u ^ hs), n) : 0u;
+    };
+    auto rnd_f = [&](int i) -> uint32_t { return Store<S>::sr ? rnd(i % C, Q + i / C) : 0u; };
 
     if constexpr (V2) {
       // this node's velocity: the reference of the flow populations it
@@ -845,8 +855,9 @@ __device__ __forceinline__ void fused_tile(
     // the receiving nodes, from the own one; mine: whether this thread has the
     // pair's flow populations. -----------------------------------------------
     const Vel<R, D>* rown = &ring[rc][eo];
+    const bool edge = (FENCE_MAPS || g.walls) && (wall_x || (D == 3 && (y == 0 || y == ny - 1)) || m == 0 || m == nm - 1);
     S* hout = b.h_out + (long long)k0 * Q * P;
-    R held[ORD && D == 2 ? KC : 1][2];    // FP32 D2Q9: summed in direction order
+    R held[ORD && D == 2 ? KC : 1][2];    // D2Q9: summed in direction order
     auto pair = [&](auto AX, int i, int j, bool mine, R cu, R cF, R cU, R fbv, int di, int dj,
                     bool bi, bool bj, int ri, int rj, auto cdot, auto PH) {
       constexpr bool axis = decltype(AX)::value;
@@ -884,27 +895,22 @@ __device__ __forceinline__ void fused_tile(
         }
         S* out = hout + (long long)q * Q * P;
         if constexpr (V2) {
-          rest[q] -= Store<S>::st_d(out + oi, pi, rnd());
-          rest[q] -= Store<S>::st_d(out + oj, pj, rnd());
+          // what the rest population makes up for: the rounding residuals
+          pi = -Store<S>::st_d(out + oi, pi, rnd(k0 + q, i));
+          pj = -Store<S>::st_d(out + oj, pj, rnd(k0 + q, j));
         } else {
-          if constexpr (RS && D == 3) {
-            rest[q] += pi;
-            rest[q] += pj;
-          }
-          if constexpr (RS && D == 2) {
-            // pairs (1, 3) (2, 4), then (5, 7) (6, 8)
-            if constexpr (half == 0) {
-              held[q][0] = pi;
-              held[q][1] = pj;
-            } else {
-              rest[q] += held[q][0];
-              rest[q] += pi;
-              rest[q] += held[q][1];
-              rest[q] += pj;
-            }
-          }
           Store<S>::st(out + oi, pi, 0u);
           Store<S>::st(out + oj, pj, 0u);
+        }
+        if constexpr (ORD && (D == 3 || half == 1)) {
+          // (2D: pairs (1, 3) (2, 4), then (5, 7) (6, 8))
+          if constexpr (D == 2) rest[q] += held[q][0];
+          rest[q] += pi;
+          if constexpr (D == 2) rest[q] += held[q][1];
+          rest[q] += pj;
+        } else if constexpr (ORD) {
+          held[q][0] = pi;
+          held[q][1] = pj;
         }
       }
       if (KG > 1 && !mine) return;
@@ -917,7 +923,7 @@ __device__ __forceinline__ void fused_tile(
         const R kp = R(1) - itf;
         Store<S>::st(b.f_out + oi, kp * Store<S>::cvt(W.f[i][col]) + (ev + od), 0u);
         Store<S>::st(b.f_out + oj, kp * Store<S>::cvt(W.f[j][col]) + (ev - od), 0u);
-      } else if constexpr (ORD) {
+      } else {
         // (f^B and q, Y are even in c_i)
         const R fbi = fB_ordered<L>(i, Ad);
         const R q = __fmaf_rn(__fmul_rn(R(4.5), cu), cu, -__fmul_rn(R(1.5), uu));
@@ -928,34 +934,36 @@ __device__ __forceinline__ void fused_tile(
           const R r = __fmaf_rn(-(f - feq), itf, f);
           return __fmaf_rn(kf, __fmaf_rn(wi, Y, lF), __fmaf_rn(fbi, kB, r));
         };
-        Store<S>::st(b.f_out + oi, post(W.f[i][col], lin, linF), 0u);
-        Store<S>::st(b.f_out + oj, post(W.f[j][col], -lin, -linF), 0u);
-      } else {
-        const R lin = w3i * cu;
-        const R ev = lam_i * p + wi * (R(4.5) * cu * cu - R(1.5) * uu);
-        const R odF = (kf * w3i) * cF;
-        R evF = (kf * wi) * (R(9) * cF * cu - R(3) * Fu);
-        if constexpr (!ORIG) evF += fbv;
         if constexpr (V2) {
-          const R eU = wi * (R(4.5) * cU * cU - R(1.5) * UU), oU = w3i * cU;
-          const R fi = Store<S>::dev_add(W.f[i][col], eU + oU);
-          const R fj = Store<S>::dev_add(W.f[j][col], eU - oU);
-          const R pi = fi - (fi - (ev + lin)) * itf + (evF + odF);
-          const R pj = fj - (fj - (ev - lin)) * itf + (evF - odF);
+          // velocity part of the equilibrium in direction +-c, from c.v, v.v
+          auto evel = [&](R c, R vv, bool plus) -> R {
+            const R qv = __fmul_rn(wi, __fmaf_rn(__fmul_rn(R(4.5), c), c, -__fmul_rn(R(1.5), vv)));
+            return __fmaf_rn(w3i, plus ? c : -c, qv);
+          };
+          const R pi = post(Store<S>::dev_add(W.f[i][col], evel(cU, UU, true)), lin, linF);
+          const R pj = post(Store<S>::dev_add(W.f[j][col], evel(cU, UU, false)), -lin, -linF);
           // scaled deviation from e(u) of the receiving node (through a wall:
           // of this node, in the reversed direction)
           auto dev = [&](bool fwd, bool bounced, int r, R post) -> R {
             const Vel<R, D> t = rown[WALLS && bounced ? 0 : r];
             R ud2;
             if constexpr (D == 3) ud2 = t.v[3];
-            else ud2 = t.v[0] * t.v[0] + t.v[1] * t.v[1];
+            else ud2 = __fmaf_rn(t.v[0], t.v[0], __fmul_rn(t.v[1], t.v[1]));
             const R c = cdot(t);
-            const R l = w3i * c, e = wi * (R(4.5) * c * c - R(1.5) * ud2);
             const bool plus = fwd != (WALLS && bounced);
-            return R(Store<S>::KF) * (post - (plus ? e + l : e - l));
+            if (WALLS && edge) {
+              // (nodes next to a boundary of a walled grid round the sum of
+              // the two parts the other way round)
+              const R qv = __fmaf_rn(__fmul_rn(R(4.5), c), c, -__fmul_rn(R(1.5), ud2));
+              return R(Store<S>::KF) * (post - __fmaf_rn(wi, qv, __fmul_rn(w3i, plus ? c : -c)));
+            }
+            return R(Store<S>::KF) * (post - evel(c, ud2, plus));
           };
-          Store<S>::st(b.f_out + oi, dev(true, bi, ri, pi), rnd());
-          Store<S>::st(b.f_out + oj, dev(false, bj, rj, pj), rnd());
+          Store<S>::st(b.f_out + oi, dev(true, bi, ri, pi), rnd_f(i));
+          Store<S>::st(b.f_out + oj, dev(false, bj, rj, pj), rnd_f(j));
+        } else {
+          Store<S>::st(b.f_out + oi, post(W.f[i][col], lin, linF), 0u);
+          Store<S>::st(b.f_out + oj, post(W.f[j][col], -lin, -linF), 0u);
         }
       }
     };
@@ -1034,24 +1042,24 @@ __device__ __forceinline__ void fused_tile(
     if (KG == 1 || kg == KG - 1) {
       const R lam0 = R(p_coef<L, R>(0));
       R f0;
-      if constexpr (V2) f0 = Store<S>::dev_add(W.f[0][col], R(-1.5 * w0) * UU);
+      if constexpr (V2) f0 = Store<S>::dev_add(W.f[0][col], R(w0) * -(R(1.5) * UU));
       else f0 = Store<S>::cvt(W.f[0][col]);
       R post;
+      const R e0 = R(w0) * -(R(1.5) * uu);
       if constexpr (ORD) {
-        const R feq = __fmaf_rn(lam0, p, __fmul_rn(R(w0), -__fmul_rn(R(1.5), uu)));
+        const R feq = __fmaf_rn(lam0, p, e0);
         const R r = __fmaf_rn(-(f0 - feq), itf, f0);
         post = __fmaf_rn(kf, __fmul_rn(R(w0), -__fmul_rn(R(3), Fu)),
                          __fmaf_rn(fB_ordered<L>(0, Ad), kB, r));
-      } else {
-        const R e0 = R(-1.5 * w0) * uu;
-        post = f0 - (f0 - (lam0 * p + e0)) * itf + (kf * (R(-3.0 * w0) * Fu) + fb.q0);
         if constexpr (V2) post = R(Store<S>::KF) * (post - e0);
+      } else {
+        post = f0 - (f0 - (lam0 * p + e0)) * itf + (kf * (R(-3.0 * w0) * Fu) + fb.q0);
       }
-      Store<S>::st(b.f_out + s, post, rnd());
+      Store<S>::st(b.f_out + s, post, rnd_f(0));
     }
 #pragma unroll
     for (int q = 0; q < KC; ++q) {
-      if constexpr (V2) h_ext<L>(b.h_out, P)[(uint32_t)(k0 + q) * P32 + s] = float(rest[q]);
+      if constexpr (V2) h_ext<L>(b.h_out, P)[(uint32_t)(k0 + q) * P32 + s] = h0p[q] + rest[q];
       else if constexpr (RS) Store<S>::st(hout + (long long)q * Q * P + s, own[q] - rest[q], 0u);
       else Store<S>::st(hout + (long long)q * Q * P + s, rest[q], 0u);
     }

@@ -360,6 +360,17 @@ __device__ __forceinline__ uint32_t lcg_next(uint32_t& r) {
   return r;
 }
 
+// the sequence's value n steps on (n a constant: one multiply-add)
+__device__ __forceinline__ uint32_t lcg_at(uint32_t r, int n) {
+  uint32_t a = 1u, c = 0u;
+#pragma unroll
+  for (int t = 0; t < n; ++t) {
+    a *= 1664525u;
+    c = c * 1664525u + 1013904223u;
+  }
+  return a * r + c;
+}
+
 // ---------------------------------------------------------------------------
 // Launch-time description of a grid and of the physics of a step.
 // ---------------------------------------------------------------------------
