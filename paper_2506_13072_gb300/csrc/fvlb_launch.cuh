@@ -175,22 +175,44 @@ struct StepShape {
                                         : (SMALL ? (B == 8 ? 3 : 4) : (B == 2 ? 4 : (B == 8 ? 3 : 2)));
 };
 
-// Planes per block along the march axis, for `tiles` tiles of a plane, `nm`
-// planes and `slots` resident blocks.  A block's time is its planes plus the
-// prologue (three planes of the velocity ring and the first copies, about
-// kPrologue planes); the grid takes blocks / slots such times, rounded up
-// while the waves are few.
-inline int pick_chunk(long long tiles, int nm, long long slots, double* cost_out = nullptr) {
-  constexpr double kPrologue = 2.5;
+// Planes per block along the march axis, from a model of the launch, fitted
+// on GB300 to chunks of 1 to 24 planes of 16 grids.  With k blocks on an SM a
+// plane takes slope k + lat (in units of one block's share of a busy SM): more
+// blocks share its throughput, one alone leaves part of it idle.
+//  - One wave (every block resident): the fullest SM's blocks and a prologue
+//    of 1.5 planes.
+//  - More: all planes and the prologues' work (`pro` planes a block) at the
+//    full SM's rate, and a share of one block's time for the uneven end.
+// us per step, this rule and the one before it (the fewest planes that still
+// fill the last wave, 2.5 planes a prologue): 64^2 FP64 6.2 / 10.2, 8x128
+// FP32 2.3 / 2.6, 100^3 FP32 215 / 223, 161x97x65 234 / 253, 64^3 FP64
+// 476 / 519, 128^3 FP16 348 / 356.
+struct ChunkModel {
+  double slope, lat, pro, tail;
+};
+template <class L, class S, bool SMALL>
+constexpr ChunkModel chunk_model() {
+  constexpr bool f64 = L::D == 3 && sizeof(S) == 8;
+  return {SMALL ? 0.6 : 1.0, L::D == 3 && !f64 ? 2.0 : 1.0,
+          f64 ? 0.3 : (L::D == 3 && sizeof(S) == 2 ? 1.2 : 0.6),
+          f64 ? 0.8 : (sizeof(S) == 2 ? 0.25 : 0.5)};
+}
+inline int pick_chunk(long long tiles, int nm, int sms, int minb, const ChunkModel& cm,
+                      double* cost_out = nullptr) {
+  constexpr double kPrologue = 1.5;
   constexpr int kMost = 32;
   const int least = (nm + 65534) / 65535;   // the chunks are the grid's z extent
   int best = least;
   double cost = 1e300;
   for (int c = least; c <= std::max(least, std::min(nm, kMost)); ++c) {
     const long long blocks = tiles * ((nm + c - 1) / c);
-    double w = (double)blocks / (double)slots;
-    w = w < 4.0 ? std::ceil(w) : w + 0.5;
-    const double t = w * (c + kPrologue);
+    const double full = cm.slope * minb + cm.lat;
+    double t;
+    if (blocks <= (long long)sms * minb)
+      t = (c + kPrologue) * (cm.slope * (double)((blocks + sms - 1) / sms) + cm.lat);
+    else
+      t = ((double)tiles * nm + (double)blocks * cm.pro) / sms * full / minb +
+          cm.tail * (c + kPrologue) * full;
     if (t <= cost) {
       cost = t;
       best = c;
@@ -218,7 +240,8 @@ cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, int threads, size_t smem, 
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-template <class L, class S, int GX, int KG, int MINB, bool WALLS, bool PADDED, bool CL, bool ORIG>
+template <class L, class S, bool SMALL, int GX, int KG, int MINB, bool WALLS, bool PADDED, bool CL,
+          bool ORIG>
 cudaError_t launch_kernel(const StepDesc& d, const Grid& g, const Phys<RT<S>>& ph,
                           const Bufs<S>& b) {
   using Sh = FusedShape<L, S, GX, KG>;
@@ -233,7 +256,8 @@ cudaError_t launch_kernel(const StepDesc& d, const Grid& g, const Phys<RT<S>>& p
   if (pl.kern != reinterpret_cast<const void*>(kern)) {
     const cudaError_t e = allow_dynamic_smem(kern, sizeof(typename Cfg::Smem));
     if (e != cudaSuccess) return e;
-    pl.mchunk = pick_chunk((long long)bx * by, nm, (long long)std::max(d.sms, 1) * MINB);
+    pl.mchunk = pick_chunk((long long)bx * by, nm, std::max(d.sms, 1), MINB,
+                           chunk_model<L, S, SMALL>());
     pl.mapped[0] = pl.mapped[1] = -1;
     pl.kern = reinterpret_cast<const void*>(kern);
   }
@@ -248,13 +272,13 @@ cudaError_t launch_kernel(const StepDesc& d, const Grid& g, const Phys<RT<S>>& p
 
 // The kernel variant of a grid: row starts on 16-byte boundaries need no
 // padded stage; padded tiles serve walled and periodic grids alike.
-template <class L, class S, int GX, int KG, int MINB, bool CL, bool ORIG>
+template <class L, class S, bool SMALL, int GX, int KG, int MINB, bool CL, bool ORIG>
 cudaError_t launch_fused(const StepDesc& d, const Grid& g, const Phys<RT<S>>& ph,
                          const Bufs<S>& b) {
   if (d.nx % (16 / (int)sizeof(S)))
-    return launch_kernel<L, S, GX, KG, MINB, true, true, CL, ORIG>(d, g, ph, b);
-  if (d.walls) return launch_kernel<L, S, GX, KG, MINB, true, false, CL, ORIG>(d, g, ph, b);
-  return launch_kernel<L, S, GX, KG, MINB, false, false, CL, ORIG>(d, g, ph, b);
+    return launch_kernel<L, S, SMALL, GX, KG, MINB, true, true, CL, ORIG>(d, g, ph, b);
+  if (d.walls) return launch_kernel<L, S, SMALL, GX, KG, MINB, true, false, CL, ORIG>(d, g, ph, b);
+  return launch_kernel<L, S, SMALL, GX, KG, MINB, false, false, CL, ORIG>(d, g, ph, b);
 }
 
 // The fused step.  ORIG: the original scheme's step (div tau_p from ph.fdiv in
@@ -265,25 +289,24 @@ cudaError_t fused_step(const StepDesc& d, const Grid& g, const Phys<RT<S>>& ph,
   using Big = StepShape<L, S, false>;
   using Small = StepShape<L, S, true>;
   if constexpr (std::is_same<S, float>::value && !ORIG) {
-    if (d.mlp) return launch_fused<L, S, Big::GX, (L::D == 3 ? 2 : 1), 2, true, false>(d, g, ph, b);
+    if (d.mlp) return launch_fused<L, S, false, Big::GX, (L::D == 3 ? 2 : 1), 2, true, false>(d, g, ph, b);
   }
   if constexpr (Big::GX != Small::GX) {
     const int by = L::D == 3 ? d.ny : 1, nm = L::D == 3 ? g.nz : d.ny;
-    auto cost = [&](int gx, int minb) {
-      double c;
-      pick_chunk((long long)((d.nx + 32 * gx - 1) / (32 * gx)) * by, nm,
-                 (long long)std::max(d.sms, 1) * minb, &c);
-      return c;
-    };
     int small = d.plan ? d.plan->small : -1;
     if (small < 0) {
-      small = cost(Small::GX, Small::MINB) < cost(Big::GX, Big::MINB);
+      auto tiles = [&](int gx) { return (long long)((d.nx + 32 * gx - 1) / (32 * gx)) * by; };
+      double cs, cb;
+      const int sms = std::max(d.sms, 1);
+      pick_chunk(tiles(Small::GX), nm, sms, Small::MINB, chunk_model<L, S, true>(), &cs);
+      pick_chunk(tiles(Big::GX), nm, sms, Big::MINB, chunk_model<L, S, false>(), &cb);
+      small = cs < cb;
       if (d.plan) d.plan->small = small;
     }
     if (small)
-      return launch_fused<L, S, Small::GX, Small::KG, Small::MINB, false, ORIG>(d, g, ph, b);
+      return launch_fused<L, S, true, Small::GX, Small::KG, Small::MINB, false, ORIG>(d, g, ph, b);
   }
-  return launch_fused<L, S, Big::GX, Big::KG, Big::MINB, false, ORIG>(d, g, ph, b);
+  return launch_fused<L, S, false, Big::GX, Big::KG, Big::MINB, false, ORIG>(d, g, ph, b);
 }
 
 template <class L, class S>
