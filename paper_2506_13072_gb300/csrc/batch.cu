@@ -1,4 +1,4 @@
-// batch.cu -- C ABI of the batched persistent step (fvlb_batch_* in fvlb.h):
+// batch.cu -- C ABI of the batched step (fvlb_batch_* in fvlb.h):
 // many independent D2Q9 grids of uneven size and parameters advanced by one
 // kernel launch per step, the steps replayed from a captured CUDA graph, and
 // the tile shape chosen by timing the candidates on the batch itself.
@@ -19,7 +19,6 @@
 namespace fvlb {
 #define FVLB_EXTERN_BATCH(S)                                                             \
   extern template cudaError_t batch_step_impl<S>(const BatchLaunch&);                    \
-  extern template int batch_occupancy_impl<S>(int);                                      \
   extern template void batch_maps_impl<S>(StageMaps*, int, const void*, const void*,     \
                                           const void*, long long);                                      \
   extern template void batch_inst_fill_impl<S>(void*, int, int, int, long long, double,  \
@@ -39,15 +38,6 @@ cudaError_t batch_step(const BatchLaunch& d) {
     case kFP16Dev: return batch_step_impl<__half>(d);
     case kBF16Dev: return batch_step_impl<__nv_bfloat16>(d);
     default: return cudaErrorInvalidValue;
-  }
-}
-
-int batch_occupancy(int storage, int gx) {
-  switch (storage) {
-    case kFP64: return batch_occupancy_impl<double>(gx);
-    case kFP32: return batch_occupancy_impl<float>(gx);
-    case kFP16Dev: return batch_occupancy_impl<__half>(gx);
-    default: return batch_occupancy_impl<__nv_bfloat16>(gx);
   }
 }
 
@@ -86,11 +76,6 @@ void batch_inst_fill(int storage, void* dst, int nx, int ny, int walls, long lon
 #undef FILL
 }
 
-cudaError_t batch_advance(long long* t, cudaStream_t stream) {
-  k_advance_step<<<1, 1, 0, stream>>>(t);
-  return cudaGetLastError();
-}
-
 }  // namespace fvlb
 
 using namespace fvlb;
@@ -125,7 +110,7 @@ struct fvlb_batch_s {
   long long t = 0;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  int gx = 4, mchunk = 16, ntiles = 0, blocks = 0, maps_gx = 0;
+  int gx = 4, mchunk = 16, ntiles = 0, maps_gx = 0;
   bool tuned = false;
   double tuned_ms = 0.0;
   cudaGraphExec_t graph = nullptr;
@@ -211,11 +196,6 @@ int upload_tiles(fvlb_batch_t b, int gx, int mchunk) {
   b->gx = gx;
   b->mchunk = mchunk;
   b->ntiles = (int)tl.size();
-  int dev = 0, sms = 1;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int per = batch_occupancy(b->storage, gx);
-  b->blocks = sms * (per > 0 ? per : 1);
   if (b->graph) {
     cudaGraphExecDestroy(b->graph);
     b->graph = nullptr;
@@ -239,7 +219,6 @@ BatchLaunch make_launch(fvlb_batch_t b) {
   d.first = b->first;
   d.tstep = b->tdev;
   d.mchunk = b->mchunk;
-  d.blocks = b->blocks;
   d.maps = b->maps + (size_t)b->parity * b->count;
   d.stream = b->stream;
   return d;
@@ -249,7 +228,6 @@ BatchLaunch make_launch(fvlb_batch_t b) {
 int direct_step(fvlb_batch_t b) {
   BatchLaunch d = make_launch(b);
   cudaError_t e = batch_step(d);
-  if (e == cudaSuccess) e = batch_advance(b->tdev, b->stream);
   if (e != cudaSuccess) return bfail(b, FVLB_ECUDA, std::string("batched step: ") + cudaGetErrorString(e));
   b->parity ^= 1;
   b->first = 0;
@@ -270,8 +248,7 @@ int build_graph(fvlb_batch_t b) {
     d.maps = b->maps + (size_t)d.parity * b->count;
     d.first = 0;
     if (e == cudaSuccess) e = batch_step(d);
-    if (e == cudaSuccess) e = batch_advance(b->tdev, b->stream);
-  }
+    }
   cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
   if (e == cudaSuccess) e = e2;
   if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph, g, 0);
@@ -425,7 +402,7 @@ int fvlb_batch_create(fvlb_batch_t* out, int lattice, int count, const fvlb_inst
   b->tiles_cap = (int)make_tiles(b, 1, 8).size();
   b->tiles = balloc(b, sizeof(BatchTile) * b->tiles_cap);
   b->maps = static_cast<StageMaps*>(balloc(b, sizeof(StageMaps) * 2 * (size_t)count));
-  b->tdev = static_cast<long long*>(balloc(b, sizeof(long long)));
+  b->tdev = static_cast<long long*>(balloc(b, 2 * sizeof(long long)));
   b->fbuf = static_cast<double*>(balloc(b, sizeof(double) * 6 * b->Nmax));
   if (!b->fA || !b->fB || !b->hA || !b->hB || !b->chi || !b->inst || !b->tiles || !b->maps || !b->tdev ||
       !b->fbuf || (b->tab_total && !b->tables)) {
@@ -465,7 +442,7 @@ int fvlb_batch_create(fvlb_batch_t* out, int lattice, int count, const fvlb_inst
       e = cudaMemcpy(b->tables, tf.data(), 4 * tf.size(), cudaMemcpyHostToDevice);
     }
   }
-  if (e == cudaSuccess) e = cudaMemset(b->tdev, 0, sizeof(long long));
+  if (e == cudaSuccess) e = cudaMemset(b->tdev, 0, 2 * sizeof(long long));
   if (e != cudaSuccess) {
     bfree_all(b);
     cudaStreamDestroy(b->stream);

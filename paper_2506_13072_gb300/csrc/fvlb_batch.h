@@ -1,4 +1,4 @@
-// fvlb_batch.h -- host-side launch interface of the batched persistent step
+// fvlb_batch.h -- host-side launch interface of the batched step
 // (internal; the public interface is the fvlb_batch_* part of fvlb.h).
 #pragma once
 
@@ -6,9 +6,9 @@
 
 namespace fvlb {
 
-// One launch of k_step_batched<D2Q9, S, gx> over `ntiles` tiles.  `inst` and
-// `tiles` are device arrays built by the host (BatchInst<S>, BatchTile);
-// blocks = 0 asks for one block per resident slot of the GPU.
+// One launch of k_step_batched<D2Q9, S, gx>, one block for each of `ntiles`
+// tiles.  `inst` and `tiles` are device arrays built by the host
+// (BatchInst<S>, BatchTile); tstep[2] is the step count (see the kernel).
 struct BatchLaunch {
   int storage;
   int gx;
@@ -17,17 +17,13 @@ struct BatchLaunch {
   int ntiles;
   void *fA, *fB, *hA, *hB, *chi;
   int parity, first;
-  const long long* tstep;
+  long long* tstep;
   int mchunk;
-  int blocks;
   const void* maps;   // device array of StageMaps, one per instance (null: no bulk copies)
   cudaStream_t stream;
 };
 
 cudaError_t batch_step(const BatchLaunch& d);
-cudaError_t batch_advance(long long* t, cudaStream_t stream);
-// resident blocks per SM of k_step_batched for (storage, gx)
-int batch_occupancy(int storage, int gx);
 // size in bytes of BatchInst<S> for the storage, and a host-side builder
 size_t batch_inst_size(int storage);
 // Fill the BatchInst of instance i into host buffer dst (batch_inst_size

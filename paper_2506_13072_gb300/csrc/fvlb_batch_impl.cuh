@@ -7,12 +7,14 @@
 
 namespace fvlb {
 
-// Resident blocks per SM: at most 18 warps, so that the loop over tiles keeps
-// its state in registers (FP64: as its stage buffers allow).
+// Threads per node and resident blocks per SM (registers and stage buffers
+// are budgeted for them).  FP16, 96 grids, us per step: 12 / GX blocks 198,
+// 8 / GX 205, 16 / GX 199, 20 / GX 212; FP32: 8 / GX 216, 4 / GX 263,
+// 12 / GX 219.
 template <class S, int GX>
 struct BatchMinB {
   static constexpr int KG = sizeof(S) == 8 ? 3 : 1;
-  static constexpr int value = sizeof(S) == 8 ? 4 / GX : 18 * 32 / FusedShape<D2Q9, S, GX, KG>::NT;
+  static constexpr int value = (sizeof(S) == 8 ? 4 : (sizeof(S) == 2 ? 12 : 8)) / GX;
 };
 template <class S, int GX>
 using BatchCfg = TileCfg<D2Q9, S, GX, BatchMinB<S, GX>::KG, BatchMinB<S, GX>::value, true, false>;
@@ -25,20 +27,11 @@ cudaError_t batch_launch_gx(const BatchLaunch& d) {
   auto kern = k_step_batched<D2Q9, S, GX, BatchMinB<S, GX>::KG, BatchMinB<S, GX>::value>;
   const cudaError_t e = allow_dynamic_smem(kern, dyn);
   if (e != cudaSuccess) return e;
-  int blocks = d.blocks;
-  if (blocks <= 0) {
-    int dev = 0, sms = 1, per = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, NT, dyn);
-    blocks = sms * (per > 0 ? per : 1);
-  }
-  kern<<<blocks, NT, dyn, d.stream>>>(
-      static_cast<const BatchInst<S>*>(d.inst), static_cast<const BatchTile*>(d.tiles),
-      d.ntiles, static_cast<S*>(d.fA), static_cast<S*>(d.fB), static_cast<S*>(d.hA),
-      static_cast<S*>(d.hB), static_cast<X*>(d.chi), d.parity, d.first, d.tstep, d.mchunk,
-      static_cast<const StageMaps*>(d.maps));
-  return cudaGetLastError();
+  return launch_pdl(kern, dim3(d.ntiles), NT, dyn, d.stream, static_cast<const BatchInst<S>*>(d.inst),
+                    static_cast<const BatchTile*>(d.tiles), static_cast<S*>(d.fA),
+                    static_cast<S*>(d.fB), static_cast<S*>(d.hA), static_cast<S*>(d.hB),
+                    static_cast<X*>(d.chi), d.parity, d.first, d.tstep, d.mchunk,
+                    static_cast<const StageMaps*>(d.maps));
 }
 
 template <class S>
@@ -48,25 +41,6 @@ cudaError_t batch_step_impl(const BatchLaunch& d) {
     case 2: return batch_launch_gx<S, 2>(d);
     case 4: return batch_launch_gx<S, 4>(d);
     default: return cudaErrorInvalidValue;
-  }
-}
-
-template <class S, int GX>
-int batch_occupancy_gx() {
-  auto kern = k_step_batched<D2Q9, S, GX, BatchMinB<S, GX>::KG, BatchMinB<S, GX>::value>;
-  constexpr size_t dyn = sizeof(typename BatchCfg<S, GX>::Smem);
-  if (allow_dynamic_smem(kern, dyn) != cudaSuccess) return 0;
-  int per = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, FusedShape<D2Q9, S, GX, BatchMinB<S, GX>::KG>::NT, dyn);
-  return per;
-}
-
-template <class S>
-int batch_occupancy_impl(int gx) {
-  switch (gx) {
-    case 1: return batch_occupancy_gx<S, 1>();
-    case 2: return batch_occupancy_gx<S, 2>();
-    default: return batch_occupancy_gx<S, 4>();
   }
 }
 

@@ -416,9 +416,6 @@ __device__ __forceinline__ void collide_site(const Grid& g, const Phys<RT<S>>& p
 
 namespace fvlb {
 
-// t += 1 on the device (one thread), after a batched step
-static __global__ void k_advance_step(long long* t) { *t += 1; }
-
 // ---------------------------------------------------------------------------
 // Original scheme (Sec. 1, Tables 1-2): the polymer stress of every node in
 // a working array tau_p[C][pitch], then its divergence by finite
