@@ -110,10 +110,13 @@ struct TileCfg {
       (unsigned)(BX * ((C * (Q - H0) + Q) * (int)sizeof(S) + C * (int)sizeof(X) +
                        (V2 ? (C + D) * 4 : 0)));
   using CLS = typename std::conditional<CL, ClosureSmem<GX, C>, NoClosureSmem>::type;
-  // exchange of a node's A - I and partial pressure sums between its threads
-  static constexpr int CP = C == 6 ? 8 : 4;
+  // Exchange of a node's A - I and partial pressure sums between its threads:
+  // thread kg's KC of each.  A record of 2 C values (FP32 3D: 48 bytes) puts
+  // eight neighbouring nodes' 16-byte pieces in different banks; the records
+  // of 16 values that this replaces cost 28 % of a 16-bit step's shared-memory
+  // wavefronts (us per step: 128^3 FP16 353 / 296, 256^3 FP32 2943 / 2901)
   struct alignas(16) Exchange {
-    R Ad[CP], pf[CP];
+    R v[KG][2 * (C / KG)];
   };
   static constexpr int NEX = KG > 1 ? Sh::TXS : 1;
   // MINB blocks per SM share 227 KB (1 KB per block is the system's)
@@ -573,11 +576,11 @@ __device__ __forceinline__ void fused_tile(
           sumf += pf[k];
         }
       } else {
-        auto& ex = sm.ex[tx];
+        auto& ex = sm.ex[tx].v[kg];
 #pragma unroll
         for (int q = 0; q < KC; ++q) {
-          ex.Ad[k0 + q] = own[q];
-          ex.pf[k0 + q] = pf[q];
+          ex[q] = own[q];
+          ex[KC + q] = pf[q];
         }
       }
     }
@@ -587,8 +590,8 @@ __device__ __forceinline__ void fused_tile(
       const auto& ex = sm.ex[tx];
 #pragma unroll
       for (int k = 0; k < C; ++k) {
-        Ad[k] = ex.Ad[k];
-        sumf += ex.pf[k];
+        Ad[k] = ex.v[k / KC][k % KC];
+        sumf += ex.v[k / KC][KC + k % KC];
       }
     }
 
