@@ -365,23 +365,36 @@ cudaError_t init_impl(const InitDesc& d) {
   return cudaGetLastError();
 }
 
+template <class L, class S, bool ORIG>
+cudaError_t launch_fields(const StepDesc& d, const Grid& g, const Phys<RT<S>>& ph, int which,
+                          double* out, const RT<S>* taup) {
+  const int threads = 128;
+  const int blocks = grid_stride_blocks(d.N, threads, d.sms);
+  const S* f = static_cast<const S*>(d.f_in);
+  const S* h = static_cast<const S*>(d.h_in);
+  switch (which) {
+    case 0: k_fields<L, S, 0, ORIG><<<blocks, threads, 0, d.stream>>>(g, ph, f, h, out, taup, d.N); break;
+    case 1: k_fields<L, S, 1, ORIG><<<blocks, threads, 0, d.stream>>>(g, ph, f, h, out, taup, d.N); break;
+    case 2: k_fields<L, S, 2><<<blocks, threads, 0, d.stream>>>(g, ph, f, h, out, taup, d.N); break;
+    default: k_fields<L, S, 3><<<blocks, threads, 0, d.stream>>>(g, ph, f, h, out, taup, d.N); break;
+  }
+  return cudaGetLastError();
+}
+
 template <class L, class S>
 cudaError_t fields_impl(const StepDesc& d, int which, double* out) {
   using R = RT<S>;
   Grid g{d.nx, d.ny, L::D == 3 ? d.nz : 1, d.walls, d.pitch};
   Phys<R> ph = make_phys<R>(d);
-  const int threads = 256;
-  const int blocks = grid_stride_blocks(d.N, threads, d.sms);
-  const S* f = static_cast<const S*>(d.f_in);
-  const S* h = static_cast<const S*>(d.h_in);
   if (d.scheme == 1) {
     R* taup = static_cast<R*>(d.taup);
-    k_taup<L, S><<<blocks, threads, 0, d.stream>>>(g, ph, h, taup, d.N);
-    k_fields<L, S, true><<<blocks, threads, 0, d.stream>>>(g, ph, f, h, which, out, taup, d.N);
-  } else {
-    k_fields<L, S><<<blocks, threads, 0, d.stream>>>(g, ph, f, h, which, out, nullptr, d.N);
+    k_taup<L, S><<<grid_stride_blocks(d.N, 256, d.sms), 256, 0, d.stream>>>(
+        g, ph, static_cast<const S*>(d.h_in), taup, d.N);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return launch_fields<L, S, true>(d, g, ph, which, out, taup);
   }
-  return cudaGetLastError();
+  return launch_fields<L, S, false>(d, g, ph, which, out, nullptr);
 }
 
 template <class L, class S>
