@@ -53,6 +53,12 @@ struct alignas(sizeof(R) * (D == 3 ? 4 : 2)) Vel {
   R v[D == 3 ? 4 : 2];
 };
 
+// A kernel's MINB: the resident blocks per SM its registers and stage buffers
+// are budgeted for, plus 100 times the most stage buffers where that is not
+// three.
+__host__ __device__ constexpr int blocks_of(int minb) { return minb % 100; }
+__host__ __device__ constexpr int stages_of(int minb) { return minb >= 100 ? minb / 100 : 3; }
+
 template <class L, class S, int GX, int KG>
 struct FusedShape {
   static_assert(L::C % KG == 0, "whole components per thread");
@@ -120,16 +126,20 @@ struct TileCfg {
   };
   static constexpr int NEX = KG > 1 ? Sh::TXS : 1;
   // MINB blocks per SM share 227 KB (1 KB per block is the system's)
-  static constexpr size_t kLimit = (size_t)(227 / MINB - 1) * 1024;
+  static constexpr size_t kLimit = (size_t)(227 / blocks_of(MINB) - 1) * 1024;
   static constexpr size_t kOther = sizeof(Vel<R, D>) * 4 * Sh::NE +
                                    sizeof(Exchange) * NEX + sizeof(CLS) + 256;
-  static constexpr int NST = kOther + 3 * sizeof(Stage) <= kLimit ? 3 : 2;
+  // stage buffers: what fits, up to stages_of(MINB)
+  static constexpr int NST =
+      stages_of(MINB) > 3 && kOther + 4 * sizeof(Stage) <= kLimit
+          ? 4
+          : (kOther + 3 * sizeof(Stage) <= kLimit ? 3 : 2);
   struct Smem {
-    alignas(128) Stage stage[NST];
-    Vel<R, D> ring[4][Sh::NE];                    // velocity of planes m-1 .. m+2
+    alignas(16) Vel<R, D> ring[4][Sh::NE];        // velocity of planes m-1 .. m+2
     Exchange ex[NEX];
     alignas(16) CLS cls;                          // learned closure (CL only)
     uint64_t bar[NST];                            // bulk-copy barriers of the stage buffers
+    alignas(128) Stage stage[NST];
   };
   static_assert(sizeof(Smem) <= kLimit, "MINB blocks must fit an SM");
 };
@@ -243,10 +253,11 @@ __device__ __forceinline__ void fused_tile(
     Vel<R, D> t;
 #pragma unroll
     for (int a = 0; a < D; ++a) t.v[a] = u[a];
-    if constexpr (D == 3) {  // |u|^2
-        if constexpr (F64) t.v[3] = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-        else t.v[3] = __fmaf_rn(u[2], u[2], __fmaf_rn(u[0], u[0], __fmul_rn(u[1], u[1])));
-      }
+    if constexpr (D == 3) {
+      // |u|^2, which the 16-bit forms ask for at 18 neighbours
+      if constexpr (V2) t.v[3] = __fmaf_rn(u[2], u[2], __fmaf_rn(u[0], u[0], __fmul_rn(u[1], u[1])));
+      else t.v[3] = R(0);
+    }
     ring[slot(q)][e] = t;
   };
   // the same from raw 16-bit populations: each enters the momentum sums
@@ -353,7 +364,8 @@ __device__ __forceinline__ void fused_tile(
     tma_load_2d(&W.chi[0][0], &tm->x, s0, 0, bar);
   };
   produce(m0);
-  if (NST > 2) produce(m0 + 1);
+#pragma unroll
+  for (int q = 1; q < NST - 1; ++q) produce(m0 + q);
   prologue();
 
   if (warp >= NCW) {
@@ -1078,7 +1090,7 @@ __device__ __forceinline__ void stage_barriers_init(uint64_t (&bar)[NST]) {
 }
 
 template <class L, class S, int GX, int KG, int MINB, bool WALLS, bool PADDED, bool CL, bool ORIG>
-__global__ void __launch_bounds__(FusedShape<L, S, GX, KG>::NT, MINB)
+__global__ void __launch_bounds__(FusedShape<L, S, GX, KG>::NT, blocks_of(MINB))
     k_step_fused(Grid g, Phys<RT<S>> ph, Bufs<S> b, int mchunk,
                  const __grid_constant__ StageMaps tm) {
   using Cfg = TileCfg<L, S, GX, KG, MINB, PADDED, CL>;
@@ -1130,7 +1142,7 @@ struct BatchTile {
 };
 
 template <class L, class S, int GX, int KG, int MINB>
-__global__ void __launch_bounds__(FusedShape<L, S, GX, KG>::NT, MINB)
+__global__ void __launch_bounds__(FusedShape<L, S, GX, KG>::NT, blocks_of(MINB))
     k_step_batched(const BatchInst<S>* __restrict__ inst, const BatchTile* __restrict__ tiles,
                    S* fA, S* fB, S* hA, S* hB, typename Store<S>::X* chi, int parity, int first,
                    long long* __restrict__ tstep, int mchunk, const StageMaps* maps) {

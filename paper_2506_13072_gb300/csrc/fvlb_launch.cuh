@@ -158,20 +158,23 @@ cudaError_t allow_dynamic_smem(K* kern, size_t bytes) {
 // MINB resident blocks per SM (registers and stage buffers are budgeted for
 // them).  Measured on GB300, MLUPS (the 256^3 / 2048^2 periodic flows; in
 // brackets the kernel with one thread per stress component):
-//   D3Q19 FP32 2,2,2: 5680 (5244); KG 1: 5517, KG 3: 5616, GX 1: 4683
-//   D3Q19 FP16 2,2,3: 6463 (4803); KG 1: 5562, MINB 2: 6188, GX 1: 4961
-//   D3Q19 FP64 (96^3) 1,2,2: 567 (343); KG 1: 371, KG 3: 540, KG 6: 430
-//   D2Q9 FP32 4,1,2: 19180 (18102); KG 3: 18223, GX 2: 19012
-//   D2Q9 FP16 4,1,4: 27500 (14835); MINB 3: 25590, 5: 23250, GX 2: 23520
-//   D2Q9 FP64 (512^2) 2,1,3: 2060 (948); KG 3: 1463, GX 4: 1968
+//   D3Q19 FP32 2,2,2: 5795 (5244); KG 1: 5480, KG 3: 5680
+//   D3Q19 FP16 2,2,3: 7110 (4803); KG 1: 5080, KG 3: 6240, MINB 2: 7130 (128^3
+//     6540 against 7120)
+//   D3Q19 FP64 (96^3) 1,2,2: 577 (343); KG 1: 366, KG 3: 550
+//   D2Q9 FP32 4,1,2: 20270 (18102); KG 3: 18223, GX 2: 19012
+//   D2Q9 FP16 4,1,4: 28200 (14835); MINB 3: 27000, 5: 23800, GX 2: 23520
+//   D2Q9 FP64 (512^2) 2,1,3: 2110 (948); KG 3: 1463, GX 4: 1968
 // SMALL: one warp's nodes per tile, for grids that leave the chip idle
-// otherwise (the larger KG spreads FP64 over the four quarters of an SM).
+// otherwise (the larger KG spreads FP64 over the four quarters of an SM; 32^3
+// FP32 1,2,4 6.9 us a step, 1,2,3 8.2, the wide tile 11.7; 48^3 FP16 1,2,5
+// 23.2, 1,2,4 25.8).
 template <class L, class S, bool SMALL>
 struct StepShape {
   static constexpr int B = sizeof(S);
   static constexpr int GX = L::D == 3 ? (SMALL || B == 8 ? 1 : 2) : (SMALL ? 1 : (B == 8 ? 2 : 4));
   static constexpr int KG = L::D == 3 ? 2 : (SMALL && B == 8 ? 3 : 1);
-  static constexpr int MINB = L::D == 3 ? (SMALL ? (B == 2 ? 4 : 3) : (B == 2 ? 3 : 2))
+  static constexpr int MINB = L::D == 3 ? (B == 8 ? 2 : (SMALL ? (B == 2 ? 5 : 4) : (B == 2 ? 3 : 2)))
                                         : (SMALL ? (B == 8 ? 3 : 4) : (B == 2 ? 4 : (B == 8 ? 3 : 2)));
 };
 
@@ -256,7 +259,7 @@ cudaError_t launch_kernel(const StepDesc& d, const Grid& g, const Phys<RT<S>>& p
   if (pl.kern != reinterpret_cast<const void*>(kern)) {
     const cudaError_t e = allow_dynamic_smem(kern, sizeof(typename Cfg::Smem));
     if (e != cudaSuccess) return e;
-    pl.mchunk = pick_chunk((long long)bx * by, nm, std::max(d.sms, 1), MINB,
+    pl.mchunk = pick_chunk((long long)bx * by, nm, std::max(d.sms, 1), blocks_of(MINB),
                            chunk_model<L, S, SMALL>());
     pl.mapped[0] = pl.mapped[1] = -1;
     pl.kern = reinterpret_cast<const void*>(kern);
@@ -305,6 +308,13 @@ cudaError_t fused_step(const StepDesc& d, const Grid& g, const Phys<RT<S>>& ph,
     }
     if (small)
       return launch_fused<L, S, true, Small::GX, Small::KG, Small::MINB, false, ORIG>(d, g, ph, b);
+  }
+  // D2Q9 FP32 with several waves of blocks: a fourth stage buffer (2048^2
+  // 206.9 us a step, 215.6 with three, 209.4 with five; with one wave it costs:
+  // 512^2 11.9 against 11.6, 517x333 10.5 against 10.1; 16-bit storage 5 %)
+  if constexpr (L::D == 2 && std::is_same<S, float>::value && !ORIG) {
+    if ((long long)d.nx * d.ny > (long long)d.sms * Big::MINB * 32 * 32 * Big::GX)
+      return launch_fused<L, S, false, Big::GX, Big::KG, 400 + Big::MINB, false, ORIG>(d, g, ph, b);
   }
   return launch_fused<L, S, false, Big::GX, Big::KG, Big::MINB, false, ORIG>(d, g, ph, b);
 }
