@@ -59,7 +59,7 @@ struct alignas(sizeof(R) * (D == 3 ? 4 : 2)) Vel {
 __host__ __device__ constexpr int blocks_of(int minb) { return minb % 100; }
 __host__ __device__ constexpr int stages_of(int minb) { return minb >= 100 ? minb / 100 : 3; }
 
-template <class L, class S, int GX, int KG>
+template <class L, class S, int GX, int KG, bool CL = false>
 struct FusedShape {
   static_assert(L::C % KG == 0, "whole components per thread");
   static constexpr int NCW = GX * KG;             // collision warps
@@ -72,7 +72,11 @@ struct FusedShape {
   static constexpr bool PAIRS = sizeof(S) == 2;
   static constexpr int PX = (EX + 2) / 2;         // pairs of a ring row
   static constexpr int NPR = EY * PX;
-  static constexpr int NFW = ((PAIRS ? NPR : NE) + 31) / 32;  // fill warps
+  // Fill warps: one slot (or pair) per thread.  The learned closure in 3D
+  // has four with two slots each: its planes take longer, and 256 threads at
+  // two blocks per SM leave 128 registers, without which the network spills
+  // (128^3, us per step: four 488, five 504, seven at 80 registers 521).
+  static constexpr int NFW = CL && L::D == 3 ? 4 : ((PAIRS ? NPR : NE) + 31) / 32;
   static constexpr int SPF = (NE + NFW * 32 - 1) / (NFW * 32);  // slots per fill thread
   static constexpr int NT = (NCW + NFW) * 32;     // threads
 };
@@ -95,7 +99,7 @@ template <class L, class S, int GX, int KG, int MINB, bool PADDED, bool CL>
 struct TileCfg {
   using R = RT<S>;
   using X = typename Store<S>::X;
-  using Sh = FusedShape<L, S, GX, KG>;
+  using Sh = FusedShape<L, S, GX, KG, CL>;
   static constexpr int D = L::D, Q = L::Q, C = L::C;
   static constexpr bool V2 = Store<S>::V2;
   static constexpr int H0 = V2 ? 1 : 0;           // first staged stress direction
@@ -171,7 +175,7 @@ __device__ __forceinline__ void fused_tile(
     StagePos& pos) {
   using R = RT<S>;
   using X = typename Store<S>::X;
-  using Sh = FusedShape<L, S, GX, KG>;
+  using Sh = FusedShape<L, S, GX, KG, CL>;
   using Cfg = TileCfg<L, S, GX, KG, MINB, PADDED, CL>;
   constexpr int D = L::D, Q = L::Q, C = L::C;
   constexpr int NCW = Sh::NCW, TXS = Sh::TXS, EX = Sh::EX, NE = Sh::NE;
@@ -506,6 +510,7 @@ __device__ __forceinline__ void fused_tile(
   const R om = ph.inv_tau_h;
   const R keep = R(1) - om;
 
+  int cl_used = 0;                      // learned closure: this warp's nodes on the network
 #pragma unroll 1
   for (int m = m0; m < m1; ++m) {
     const int st = pos.st;
@@ -726,12 +731,7 @@ __device__ __forceinline__ void fused_tile(
 #pragma unroll
         for (int c = 0; c < C; ++c) cls.chi[c][tx] = used ? nn[c] : an[c];
       }
-      const unsigned act = __ballot_sync(0xffffffffu, active && mine);
-      const unsigned use = __ballot_sync(0xffffffffu, used);
-      if (lane == 0 && ph.cl_count && act) {
-        atomicAdd(ph.cl_count, (unsigned long long)__popc(use));
-        atomicAdd(ph.cl_count + 1, (unsigned long long)__popc(act & ~use));
-      }
+      cl_used += __popc(__ballot_sync(0xffffffffu, used));
       if constexpr (KG > 1) group_sync();
       else __syncwarp();
       if (!active) continue;
@@ -1078,6 +1078,15 @@ __device__ __forceinline__ void fused_tile(
       else Store<S>::st(hout + (long long)q * Q * P + s, rest[q], 0u);
     }
   }
+  // The closure's counts, once per warp and tile: two additions per warp and
+  // plane to the same two words kept a 128^3 step 23 us longer.
+  if constexpr (CL) {
+    const unsigned act = __ballot_sync(0xffffffffu, active && (KG == 1 || (lane >> 4) == kg));
+    if (lane == 0 && ph.cl_count && act) {
+      atomicAdd(ph.cl_count, (unsigned long long)cl_used);
+      atomicAdd(ph.cl_count + 1, (unsigned long long)(__popc(act) * (m1 - m0) - cl_used));
+    }
+  }
 }
 
 // Initialise a block's stage barriers (one thread; the first copies are
@@ -1090,13 +1099,13 @@ __device__ __forceinline__ void stage_barriers_init(uint64_t (&bar)[NST]) {
 }
 
 template <class L, class S, int GX, int KG, int MINB, bool WALLS, bool PADDED, bool CL, bool ORIG>
-__global__ void __launch_bounds__(FusedShape<L, S, GX, KG>::NT, blocks_of(MINB))
+__global__ void __launch_bounds__(FusedShape<L, S, GX, KG, CL>::NT, blocks_of(MINB))
     k_step_fused(Grid g, Phys<RT<S>> ph, Bufs<S> b, int mchunk,
                  const __grid_constant__ StageMaps tm) {
   using Cfg = TileCfg<L, S, GX, KG, MINB, PADDED, CL>;
   extern __shared__ __align__(128) unsigned char fvlb_tile_smem[];
   auto& sm = *reinterpret_cast<typename Cfg::Smem*>(fvlb_tile_smem);
-  if (threadIdx.x == FusedShape<L, S, GX, KG>::NCW * 32) stage_barriers_init(sm.bar);
+  if (threadIdx.x == FusedShape<L, S, GX, KG, CL>::NCW * 32) stage_barriers_init(sm.bar);
   pdl_wait();   // nothing above reads or writes global memory
   if constexpr (CL) mlp_load(sm.cls.P, static_cast<const MlpPacked*>(ph.mlp));
   StagePos pos;
@@ -1107,7 +1116,7 @@ __global__ void __launch_bounds__(FusedShape<L, S, GX, KG>::NT, blocks_of(MINB))
   // this step: 64^2 FP64 17.3 us a step with the trigger at the start, 11.1
   // at the last plane, 11.0 here, 12.3 without; 128^2 FP32 3.75, 3.67, 3.12
   // and 6.15; 517 x 333 FP32 11.2, 11.0, 10.8 and 12.5; large grids the same.)
-  if (threadIdx.x < FusedShape<L, S, GX, KG>::NCW * 32) pdl_trigger();
+  if (threadIdx.x < FusedShape<L, S, GX, KG, CL>::NCW * 32) pdl_trigger();
 }
 
 // ---------------------------------------------------------------------------

@@ -247,7 +247,7 @@ template <class L, class S, bool SMALL, int GX, int KG, int MINB, bool WALLS, bo
           bool ORIG>
 cudaError_t launch_kernel(const StepDesc& d, const Grid& g, const Phys<RT<S>>& ph,
                           const Bufs<S>& b) {
-  using Sh = FusedShape<L, S, GX, KG>;
+  using Sh = FusedShape<L, S, GX, KG, CL>;
   using Cfg = TileCfg<L, S, GX, KG, MINB, PADDED, CL>;
   auto kern = k_step_fused<L, S, GX, KG, MINB, WALLS, PADDED, CL, ORIG>;
   const int bx = (d.nx + Sh::TXS - 1) / Sh::TXS;

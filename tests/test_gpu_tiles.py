@@ -96,3 +96,28 @@ def test_steps_in_a_captured_graph(shape, prec):
         out.append(np.concatenate([s.u().ravel(), s.A().ravel(), s.p().ravel()]))
         s.close()
     assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("shape,walls", [((131, 300), 0b10), ((33, 40), 0), ((33, 7, 4), 0),
+                                         ((66, 30, 40), 0b110), ((100, 41, 37), 0), ((64, 3, 70), 0b001)])
+def test_closure_tile_edges(shape, walls):
+    """The learned closure's tile (fill threads with two ring slots in 3D, counts
+    added up per tile): with no network value accepted it is the plain step,
+    and every node update is counted once."""
+    from paper_2506_13072_gb300 import fvlb as F
+    pr = _problem(shape, walls)
+    net = F.Mlp(pr.lattice, seed=3)
+    out = []
+    for tol in (None, 1e-12):
+        s = gpu_sim(pr, FP32)
+        if tol is not None:
+            s.set_closure(net, tol=tol)
+        s.step(7)
+        out.append((s.u(), s.A()))
+        if tol is not None:
+            st = s.closure_stats()
+            assert st["fallback"] == 7 * pr.sites and st["network"] == 0
+        s.close()
+    net.close()
+    assert rel_l2(out[1][0], out[0][0], 1e-30) <= TOL[FP32]
+    assert rel_l2(out[1][1], out[0][1], 1e-30) <= TOL[FP32]
