@@ -49,14 +49,28 @@ struct MlpParams {
   static constexpr int N = B3 + OUT;
 };
 
-// Packed inference weights (FP16 rows padded so that the 32-bit fragment
-// loads of a warp hit 32 distinct shared-memory banks) and FP32 biases.
+// Packed inference weights in the order the mma's lanes take them, and FP32
+// biases.  One 16-byte piece per lane holds four B registers: of layers 1
+// and 2 the k16 tile's (b0, b1) for two neighbouring n8 tiles, of layer 3
+// (whose 8 outputs are one n8 tile) the (b0, b1) of two k16 tiles.  A warp's
+// weights are then 22 conflict-free 16-byte loads instead of 88 4-byte ones
+// (Taylor-Green 128^3, us per step: 470 against 488; four weights at a time
+// need registers: with 80 a thread instead of 128 it was 603 against 544).
 struct __align__(16) MlpPacked {
-  __half W1[kMlpH][24];  // [n][k], k < 16 (inputs zero-padded to 16)
-  __half W2[kMlpH][72];  // [n][k], k < 64
-  __half W3[8][72];      // [n][k], n < OUT (rows beyond OUT are zero)
+  uint32_t W1[4][32][4];     // [n16 tile][lane][b0, b1 of n8 tile 0; of 1], k < 16 (inputs zero-padded)
+  uint32_t W2[4][4][32][4];  // [n16 tile][k16 tile][lane][...]
+  uint32_t W3[2][32][4];     // [k32 tile][lane][b0, b1 of k16 tile 0; of 1], outputs beyond OUT zero
   float b1[kMlpH], b2[kMlpH], b3[8];
 };
+
+// B register r (0: k = 2 t, 2 t + 1; 1: k = 2 t + 8, + 9) of lane (g, t): the
+// weights w(n = g, k) of an n8 x k16 tile
+template <class F>
+__device__ __forceinline__ uint32_t mlp_b_register(int lane, int r, F&& w) {
+  const int g = lane >> 2, k = 2 * (lane & 3) + 8 * r;
+  const __half2 v = __floats2half2_rn(w(g, k), w(g, k + 1));
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
 
 __device__ __forceinline__ uint32_t h2_bits(__half2 v) { return *reinterpret_cast<uint32_t*>(&v); }
 
@@ -91,6 +105,9 @@ __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4],
 __device__ __forceinline__ uint32_t lds32(const __half* p) {
   return *reinterpret_cast<const uint32_t*>(p);
 }
+__device__ __forceinline__ uint4 lds128(const uint32_t* p) {
+  return *reinterpret_cast<const uint4*>(p);
+}
 
 // One warp: Y[r][0..7] = MLP(X[r][0..15]) for the 16 rows r of m-tile mt
 // (rows 16 mt .. 16 mt + 15).  X and Y are shared-memory staging rows; P
@@ -114,16 +131,12 @@ __device__ __forceinline__ void mlp_tile(const MlpPacked& P, const __half (*X)[2
   uint32_t a2[4][4];
 #pragma unroll
   for (int kt = 0; kt < 4; ++kt) {
-    float h0[4], h1[4];
-    {
-      const float c0 = P.b1[2 * kt * 8 + 2 * t], c1 = P.b1[2 * kt * 8 + 2 * t + 1];
-      h0[0] = c0; h0[1] = c1; h0[2] = c0; h0[3] = c1;
-      const float d0 = P.b1[(2 * kt + 1) * 8 + 2 * t], d1 = P.b1[(2 * kt + 1) * 8 + 2 * t + 1];
-      h1[0] = d0; h1[1] = d1; h1[2] = d0; h1[3] = d1;
-    }
-    mma_16816(h0, a, lds32(&P.W1[2 * kt * 8 + g][2 * t]), lds32(&P.W1[2 * kt * 8 + g][2 * t + 8]));
-    mma_16816(h1, a, lds32(&P.W1[(2 * kt + 1) * 8 + g][2 * t]),
-              lds32(&P.W1[(2 * kt + 1) * 8 + g][2 * t + 8]));
+    const float2 c = *reinterpret_cast<const float2*>(&P.b1[2 * kt * 8 + 2 * t]);
+    const float2 d = *reinterpret_cast<const float2*>(&P.b1[(2 * kt + 1) * 8 + 2 * t]);
+    float h0[4] = {c.x, c.y, c.x, c.y}, h1[4] = {d.x, d.y, d.x, d.y};
+    const uint4 w = lds128(P.W1[kt][lane]);
+    mma_16816(h0, a, w.x, w.y);
+    mma_16816(h1, a, w.z, w.w);
     a2[kt][0] = gelu_f16x2(h0[0], h0[1]);
     a2[kt][1] = gelu_f16x2(h0[2], h0[3]);
     a2[kt][2] = gelu_f16x2(h1[0], h1[1]);
@@ -132,26 +145,25 @@ __device__ __forceinline__ void mlp_tile(const MlpPacked& P, const __half (*X)[2
   // layers 2 (64 -> 64) and 3 (64 -> 8, OUT used): each pair of layer-2
   // n-tiles is one layer-3 k-tile, accumulated as soon as it is ready
   float y[4];
-  y[0] = P.b3[2 * t]; y[1] = P.b3[2 * t + 1]; y[2] = y[0]; y[3] = y[1];
+  {
+    const float2 c = *reinterpret_cast<const float2*>(&P.b3[2 * t]);
+    y[0] = c.x; y[1] = c.y; y[2] = c.x; y[3] = c.y;
+  }
 #pragma unroll
   for (int k3 = 0; k3 < 4; ++k3) {
-    float h0[4], h1[4];
-    {
-      const float c0 = P.b2[2 * k3 * 8 + 2 * t], c1 = P.b2[2 * k3 * 8 + 2 * t + 1];
-      h0[0] = c0; h0[1] = c1; h0[2] = c0; h0[3] = c1;
-      const float d0 = P.b2[(2 * k3 + 1) * 8 + 2 * t], d1 = P.b2[(2 * k3 + 1) * 8 + 2 * t + 1];
-      h1[0] = d0; h1[1] = d1; h1[2] = d0; h1[3] = d1;
-    }
+    const float2 c = *reinterpret_cast<const float2*>(&P.b2[2 * k3 * 8 + 2 * t]);
+    const float2 d = *reinterpret_cast<const float2*>(&P.b2[(2 * k3 + 1) * 8 + 2 * t]);
+    float h0[4] = {c.x, c.y, c.x, c.y}, h1[4] = {d.x, d.y, d.x, d.y};
 #pragma unroll
     for (int kt = 0; kt < 4; ++kt) {
-      mma_16816(h0, a2[kt], lds32(&P.W2[2 * k3 * 8 + g][kt * 16 + 2 * t]),
-                lds32(&P.W2[2 * k3 * 8 + g][kt * 16 + 2 * t + 8]));
-      mma_16816(h1, a2[kt], lds32(&P.W2[(2 * k3 + 1) * 8 + g][kt * 16 + 2 * t]),
-                lds32(&P.W2[(2 * k3 + 1) * 8 + g][kt * 16 + 2 * t + 8]));
+      const uint4 w = lds128(P.W2[k3][kt][lane]);
+      mma_16816(h0, a2[kt], w.x, w.y);
+      mma_16816(h1, a2[kt], w.z, w.w);
     }
     const uint32_t a3[4] = {gelu_f16x2(h0[0], h0[1]), gelu_f16x2(h0[2], h0[3]),
                             gelu_f16x2(h1[0], h1[1]), gelu_f16x2(h1[2], h1[3])};
-    mma_16816(y, a3, lds32(&P.W3[g][k3 * 16 + 2 * t]), lds32(&P.W3[g][k3 * 16 + 2 * t + 8]));
+    const uint2 w = *reinterpret_cast<const uint2*>(&P.W3[k3 >> 1][lane][2 * (k3 & 1)]);
+    mma_16816(y, a3, w.x, w.y);
   }
   Y[r0][2 * t] = y[0];
   Y[r0][2 * t + 1] = y[1];

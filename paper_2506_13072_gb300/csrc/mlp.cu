@@ -434,17 +434,24 @@ template <int IN, int OUT>
 __global__ void k_mlp_pack(const float* __restrict__ prm, MlpPacked* __restrict__ P) {
   using PP = MlpParams<IN, OUT>;
   constexpr int H = kMlpH;
-  for (int e = threadIdx.x; e < H * 24; e += blockDim.x) {
-    const int n = e / 24, k = e % 24;
-    P->W1[n][k] = __float2half_rn(k < IN ? prm[PP::W1 + n * IN + k] : 0.f);
+  // (see MlpPacked) e = lane * 4 + register within each 128-register piece
+  for (int e = threadIdx.x; e < 4 * 128; e += blockDim.x) {
+    const int nt = e >> 7, lane = (e >> 2) & 31, q = e & 3;
+    P->W1[nt][lane][q] = mlp_b_register(lane, q & 1, [&](int g, int k) {
+      return k < IN ? prm[PP::W1 + (16 * nt + 8 * (q >> 1) + g) * IN + k] : 0.f;
+    });
   }
-  for (int e = threadIdx.x; e < H * 72; e += blockDim.x) {
-    const int n = e / 72, k = e % 72;
-    P->W2[n][k] = __float2half_rn(k < H ? prm[PP::W2 + n * H + k] : 0.f);
+  for (int e = threadIdx.x; e < 16 * 128; e += blockDim.x) {
+    const int nt = e >> 9, kt = (e >> 7) & 3, lane = (e >> 2) & 31, q = e & 3;
+    P->W2[nt][kt][lane][q] = mlp_b_register(lane, q & 1, [&](int g, int k) {
+      return prm[PP::W2 + (16 * nt + 8 * (q >> 1) + g) * H + 16 * kt + k];
+    });
   }
-  for (int e = threadIdx.x; e < 8 * 72; e += blockDim.x) {
-    const int n = e / 72, k = e % 72;
-    P->W3[n][k] = __float2half_rn(n < OUT && k < H ? prm[PP::W3 + n * H + k] : 0.f);
+  for (int e = threadIdx.x; e < 2 * 128; e += blockDim.x) {
+    const int kp = e >> 7, lane = (e >> 2) & 31, q = e & 3;
+    P->W3[kp][lane][q] = mlp_b_register(lane, q & 1, [&](int g, int k) {
+      return g < OUT ? prm[PP::W3 + g * H + 32 * kp + 16 * (q >> 1) + k] : 0.f;
+    });
   }
   for (int e = threadIdx.x; e < H; e += blockDim.x) {
     P->b1[e] = prm[PP::B1 + e];
