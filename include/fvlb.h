@@ -53,9 +53,10 @@ enum {
   FVLB_EUNSTABLE = -4, /* the diagnostics found a non-finite value */
   FVLB_ETIMEOUT = -5,  /* a bounded device wait ran out: a step kernel's staged
                         * copies did not arrive within about 2 s; the state is
-                        * invalid until fvlb_init_fields / fvlb_load_state.
-                        * Reported by fvlb_fields, fvlb_reduce and
-                        * fvlb_status(h, 1). */
+                        * invalid until fvlb_init_fields / fvlb_load_state
+                        * (a batch's: for good).  Reported by fvlb_fields,
+                        * fvlb_reduce, fvlb_status(h, 1), fvlb_batch_fields
+                        * and fvlb_batch_synchronize. */
   FVLB_ESTATE = -6     /* call not allowed in the handle's current state */
 };
 
@@ -378,7 +379,8 @@ int fvlb_batch_init_fields(fvlb_batch_t b, int index, const double *u0,
  * replay a captured two-step graph. */
 int fvlb_batch_step(fvlb_batch_t b, long n);
 
-/* One field of instance `index` (as fvlb_fields), synchronising. */
+/* One field of instance `index` (as fvlb_fields), synchronising.
+ * FVLB_ETIMEOUT (after the copy) if a step's bounded wait ran out. */
 int fvlb_batch_fields(fvlb_batch_t b, int index, int which, double *host_out,
                       size_t count);
 
@@ -388,6 +390,8 @@ int fvlb_batch_fields(fvlb_batch_t b, int index, int which, double *host_out,
 int fvlb_batch_info(fvlb_batch_t b, long long *sites, double *bytes_per_update,
                     int *gx, int *rows, double *tuned_ms_per_step);
 
+/* Wait for all GPU work of the batch; FVLB_ETIMEOUT if a step's bounded wait
+ * ran out. */
 int fvlb_batch_synchronize(fvlb_batch_t b);
 int fvlb_batch_get_time(fvlb_batch_t b, long *t);
 const char *fvlb_batch_last_error(fvlb_batch_t b);

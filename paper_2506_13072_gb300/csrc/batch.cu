@@ -20,11 +20,11 @@ namespace fvlb {
 #define FVLB_EXTERN_BATCH(S)                                                             \
   extern template cudaError_t batch_step_impl<S>(const BatchLaunch&);                    \
   extern template void batch_maps_impl<S>(StageMaps*, int, const void*, const void*,     \
-                                          const void*, long long);                                      \
+                                          const void*, long long);                       \
   extern template void batch_inst_fill_impl<S>(void*, int, int, int, long long, double,  \
                                                double, double, double, int, const double*, \
                                                double, const void*, long long, long long,  \
-                                               long long);
+                                               long long, unsigned*);
 FVLB_EXTERN_BATCH(double)
 FVLB_EXTERN_BATCH(float)
 FVLB_EXTERN_BATCH(__half)
@@ -63,10 +63,10 @@ size_t batch_inst_size(int storage) {
 void batch_inst_fill(int storage, void* dst, int nx, int ny, int walls, long long pitch,
                      double tau_f, double tau_h, double eta_p, double lambda, int force_kind,
                      const double F0[3], double omega, const void* tables, long long f_off,
-                     long long h_off, long long chi_off) {
+                     long long h_off, long long chi_off, unsigned* err) {
 #define FILL(S)                                                                             \
   batch_inst_fill_impl<S>(dst, nx, ny, walls, pitch, tau_f, tau_h, eta_p, lambda, force_kind, \
-                          F0, omega, tables, f_off, h_off, chi_off)
+                          F0, omega, tables, f_off, h_off, chi_off, err)
   switch (storage) {
     case kFP64: FILL(double); break;
     case kFP32: FILL(float); break;
@@ -74,6 +74,27 @@ void batch_inst_fill(int storage, void* dst, int nx, int ny, int walls, long lon
     default: FILL(__nv_bfloat16); break;
   }
 #undef FILL
+}
+
+// One of the step's bounded waits, as the tiles of instance i make it, on a
+// barrier that nothing arrives at.
+template <class S>
+__global__ void k_expire_wait(const BatchInst<S>* inst, int i) {
+  __shared__ uint64_t bar;
+  mbar_init(&bar, 1);
+  mbar_wait(&bar, 0, inst[i].ph.err);
+}
+
+cudaError_t batch_expire_wait(int storage, const void* inst, int i, cudaStream_t stream) {
+  switch (storage) {
+#define EXPIRE(S) k_expire_wait<S><<<1, 1, 0, stream>>>(static_cast<const BatchInst<S>*>(inst), i)
+    case kFP64: EXPIRE(double); break;
+    case kFP32: EXPIRE(float); break;
+    case kFP16Dev: EXPIRE(__half); break;
+    default: EXPIRE(__nv_bfloat16); break;
+#undef EXPIRE
+  }
+  return cudaGetLastError();
 }
 
 }  // namespace fvlb
@@ -105,6 +126,10 @@ struct fvlb_batch_s {
   StageMaps* maps = nullptr;  // [parity][instance] of the current tile width
   int tiles_cap = 0;
   long long* tdev = nullptr;
+  // Bounded device waits that ran out (bit 0: staging copies): a word of
+  // page-locked host memory that the kernels write through its device address,
+  // so that reading it after a synchronisation costs no copy.
+  volatile unsigned* waits = nullptr;
   double* fbuf = nullptr;
   int parity = 0, first = 1;
   long long t = 0;
@@ -150,6 +175,16 @@ void bfree_all(fvlb_batch_t b) {
     else cudaFree(p);
   }
   b->owned.clear();
+  if (b->waits) cudaFreeHost(const_cast<unsigned*>(b->waits));
+  b->waits = nullptr;
+}
+
+// FVLB_ETIMEOUT if a step's bounded wait ran out; the stream is synchronised.
+int wait_check(fvlb_batch_t b) {
+  if (*b->waits)
+    return bfail(b, FVLB_ETIMEOUT,
+                 "a batched step's staged copies did not arrive in time; the state is invalid");
+  return FVLB_OK;
 }
 
 // tile list of a shape: every instance's x tiles and row chunks, largest
@@ -404,6 +439,22 @@ int fvlb_batch_create(fvlb_batch_t* out, int lattice, int count, const fvlb_inst
   b->maps = static_cast<StageMaps*>(balloc(b, sizeof(StageMaps) * 2 * (size_t)count));
   b->tdev = static_cast<long long*>(balloc(b, 2 * sizeof(long long)));
   b->fbuf = static_cast<double*>(balloc(b, sizeof(double) * 6 * b->Nmax));
+  void* word = nullptr;
+  unsigned* word_dev = nullptr;
+  e = cudaHostAlloc(&word, sizeof(unsigned), cudaHostAllocMapped);
+  if (e == cudaSuccess) {
+    b->waits = static_cast<volatile unsigned*>(word);
+    *b->waits = 0;
+    e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&word_dev), word, 0);
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    bfree_all(b);
+    cudaStreamDestroy(b->stream);
+    delete b;
+    return set_global_error(e == cudaErrorMemoryAllocation ? FVLB_ENOMEM : FVLB_ECUDA,
+                            "fvlb_batch_create: page-locked host allocation failed");
+  }
   if (!b->fA || !b->fB || !b->hA || !b->hB || !b->chi || !b->inst || !b->tiles || !b->maps || !b->tdev ||
       !b->fbuf || (b->tab_total && !b->tables)) {
     bfree_all(b);
@@ -431,7 +482,7 @@ int fvlb_batch_create(fvlb_batch_t* out, int lattice, int count, const fvlb_inst
     }
     batch_inst_fill(storage, inst.data() + batch_inst_size(storage) * i, s.nx, s.ny, (int)s.walls,
                     b->pitch[i], s.tau_s, 0.501, s.eta_p, s.lambda, s.force.kind, s.force.F0,
-                    s.force.omega, tptr, b->f_off[i], b->h_off[i], b->chi_off[i]);
+                    s.force.omega, tptr, b->f_off[i], b->h_off[i], b->chi_off[i], word_dev);
   }
   e = cudaMemcpy(b->inst, inst.data(), inst.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess && b->tab_total) {
@@ -552,7 +603,7 @@ int fvlb_batch_fields(fvlb_batch_t b, int index, int which, double* host_out, si
     e = cudaMemcpyAsync(host_out, b->fbuf, sizeof(double) * b->N[index] * nc, cudaMemcpyDeviceToHost, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return bfail(b, FVLB_ECUDA, std::string("fvlb_batch_fields: ") + cudaGetErrorString(e));
-  return FVLB_OK;
+  return wait_check(b);
 }
 
 int fvlb_batch_info(fvlb_batch_t b, long long* sites, double* bytes_per_update, int* gx,
@@ -571,6 +622,16 @@ int fvlb_batch_synchronize(fvlb_batch_t b) {
   if (!b) return set_global_error(FVLB_EINVAL, "NULL batch");
   cudaError_t e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return bfail(b, FVLB_ECUDA, std::string("fvlb_batch_synchronize: ") + cudaGetErrorString(e));
+  return wait_check(b);
+}
+
+// For the tests of failure detection (not in fvlb.h): let one bounded wait of
+// instance `index` run out, without a step and within its 2 s.
+int fvlb_batch_expire_wait(fvlb_batch_t b, int index) {
+  if (!b) return set_global_error(FVLB_EINVAL, "NULL batch");
+  if (index < 0 || index >= b->count) return bfail(b, FVLB_EINVAL, "fvlb_batch_expire_wait: bad index");
+  const cudaError_t e = batch_expire_wait(b->storage, b->inst, index, b->stream);
+  if (e != cudaSuccess) return bfail(b, FVLB_ECUDA, std::string("fvlb_batch_expire_wait: ") + cudaGetErrorString(e));
   return FVLB_OK;
 }
 

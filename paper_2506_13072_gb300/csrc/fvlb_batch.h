@@ -27,10 +27,11 @@ cudaError_t batch_step(const BatchLaunch& d);
 // size in bytes of BatchInst<S> for the storage, and a host-side builder
 size_t batch_inst_size(int storage);
 // Fill the BatchInst of instance i into host buffer dst (batch_inst_size
-// bytes): grid, physics in the working precision, arena offsets, force.
+// bytes): grid, physics in the working precision, arena offsets, force, and
+// the device address of the batch's record of waits that ran out.
 void batch_inst_fill(int storage, void* dst, int nx, int ny, int walls, long long pitch,
                      double tau_f, double tau_h, double eta_p, double lambda, int force_kind,
                      const double F0[3], double omega, const void* tables, long long f_off,
-                     long long h_off, long long chi_off);
+                     long long h_off, long long chi_off, unsigned* err);
 
 }  // namespace fvlb

@@ -55,7 +55,7 @@ template <class S>
 void batch_inst_fill_impl(void* dst, int nx, int ny, int walls, long long pitch, double tau_f,
                           double tau_h, double eta_p, double lambda, int force_kind,
                           const double* F0, double omega, const void* tables, long long f_off,
-                          long long h_off, long long chi_off) {
+                          long long h_off, long long chi_off, unsigned* err) {
   using R = RT<S>;
   BatchInst<S> I{};
   I.g = Grid{nx, ny, 1, walls, pitch};
@@ -70,6 +70,7 @@ void batch_inst_fill_impl(void* dst, int nx, int ny, int walls, long long pitch,
   sd.four_roll = force_kind == 2;
   sd.amp = F0[0];
   sd.tables = tables;
+  sd.err = err;
   for (int a = 0; a < 3; ++a) sd.Fv[a] = force_kind == 1 ? F0[a] : 0.0;
   I.ph = make_phys<R>(sd);
   I.f_off = f_off;

@@ -6,5 +6,5 @@ template cudaError_t batch_step_impl<__nv_bfloat16>(const BatchLaunch&);
 template void batch_maps_impl<__nv_bfloat16>(StageMaps*, int, const void*, const void*, const void*, long long);
 template void batch_inst_fill_impl<__nv_bfloat16>(void*, int, int, int, long long, double, double, double,
                                        double, int, const double*, double, const void*, long long,
-                                       long long, long long);
+                                       long long, long long, unsigned*);
 }  // namespace fvlb
