@@ -436,7 +436,9 @@ int fvlb_mlp_get_params(fvlb_mlp_t m, float *host, size_t count);
 int fvlb_mlp_set_params(fvlb_mlp_t m, const float *host, size_t count);
 
 /* Gradient of the loss over n host pairs, computed by the training kernels
- * (FP32), and the loss. */
+ * (FP32), and the loss.  The network keeps the device memory of the samples
+ * for its next fvlb_mlp_grad or fvlb_mlp_infer, at most that of 262144 of
+ * them (22 MB in 3D, 12 MB in 2D); a larger inference gives its back. */
 int fvlb_mlp_grad(fvlb_mlp_t m, const float *x, const float *y, long n, float *grad,
                   double *loss);
 

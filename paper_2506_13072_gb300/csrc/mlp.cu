@@ -505,8 +505,8 @@ struct fvlb_mlp_s {
   fvlb_alloc_fn alloc = nullptr;
   fvlb_free_fn free_ = nullptr;
   void* actx = nullptr;
-  // samples of fvlb_mlp_grad / _infer on the device, kept from call to call
-  // (grown to the largest one, given back with the network)
+  // samples of fvlb_mlp_grad / _infer on the device, kept from call to call:
+  // grown to the largest one within keep_floats, given back with the network
   float* stage = nullptr;
   size_t stage_floats = 0;
   std::vector<void*> owned;
@@ -533,17 +533,29 @@ void* malloc_dev(fvlb_mlp_t m, size_t bytes) {
   return p;
 }
 
-float* stage_of(fvlb_mlp_t m, size_t floats) {
-  if (floats <= m->stage_floats) return m->stage;
-  if (m->stage) {
-    cudaStreamSynchronize(m->stream);
-    m->owned.erase(std::find(m->owned.begin(), m->owned.end(), static_cast<void*>(m->stage)));
-    if (m->free_) m->free_(m->stage, m->actx);
-    else cudaFree(m->stage);
+void free_dev(fvlb_mlp_t m, void* p) {
+  m->owned.erase(std::find(m->owned.begin(), m->owned.end(), p));
+  if (m->free_) m->free_(p, m->actx);
+  else cudaFree(p);
+}
+
+// Samples a network may keep between calls: those of the largest gradient
+// (22 MB in 3D).  Inference takes any number.
+size_t keep_floats(fvlb_mlp_t m) { return (size_t)(m->IN + m->OUT) * kMaxBatches * kTB; }
+
+// The device buffer for a call's samples, and its return at the call's end
+// (the stream is idle): a larger one than may be kept is freed.
+float* stage_take(fvlb_mlp_t m, size_t floats) {
+  if (floats > keep_floats(m)) return static_cast<float*>(malloc_dev(m, sizeof(float) * floats));
+  if (floats > m->stage_floats) {
+    if (m->stage) free_dev(m, m->stage);
+    m->stage = static_cast<float*>(malloc_dev(m, sizeof(float) * floats));
+    m->stage_floats = m->stage ? floats : 0;
   }
-  m->stage = static_cast<float*>(malloc_dev(m, sizeof(float) * floats));
-  m->stage_floats = m->stage ? floats : 0;
   return m->stage;
+}
+void stage_give(fvlb_mlp_t m, float* p) {
+  if (p != m->stage) free_dev(m, p);
 }
 
 // blocks of a gradient over n samples
@@ -768,7 +780,7 @@ int fvlb_mlp_train(fvlb_mlp_t m, long steps, int batch, double lr, double* last_
 int fvlb_mlp_grad(fvlb_mlp_t m, const float* x, const float* t, long n, float* grad, double* loss) {
   if (!m || !x || !t || !grad || n < 1) return mfail(m, FVLB_EINVAL, "fvlb_mlp_grad: bad arguments");
   if ((n + kTB - 1) / kTB > kMaxBatches) return mfail(m, FVLB_EINVAL, "fvlb_mlp_grad: too many samples");
-  float* dx = stage_of(m, (size_t)(m->IN + m->OUT) * (size_t)n);
+  float* dx = stage_take(m, (size_t)(m->IN + m->OUT) * (size_t)n);
   if (!dx) return mfail(m, FVLB_ENOMEM, "fvlb_mlp_grad: device allocation failed");
   float* dt = dx + (size_t)m->IN * n;
   cudaError_t e = cudaMemcpyAsync(dx, x, sizeof(float) * m->IN * n, cudaMemcpyHostToDevice, m->stream);
@@ -783,13 +795,15 @@ int fvlb_mlp_grad(fvlb_mlp_t m, const float* x, const float* t, long n, float* g
   if (e == cudaSuccess) e = cudaMemcpyAsync(grad, m->grad, sizeof(float) * m->NP, cudaMemcpyDeviceToHost, m->stream);
   if (e == cudaSuccess && loss) e = cudaMemcpyAsync(loss, m->loss, sizeof(double), cudaMemcpyDeviceToHost, m->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
+  else cudaStreamSynchronize(m->stream);
+  stage_give(m, dx);
   if (e != cudaSuccess) return mfail(m, FVLB_ECUDA, std::string("fvlb_mlp_grad: ") + cudaGetErrorString(e));
   return FVLB_OK;
 }
 
 int fvlb_mlp_infer(fvlb_mlp_t m, const float* x, long n, float* y) {
   if (!m || !x || !y || n < 1) return mfail(m, FVLB_EINVAL, "fvlb_mlp_infer: bad arguments");
-  float* dx = stage_of(m, (size_t)(m->IN + m->OUT) * (size_t)n);
+  float* dx = stage_take(m, (size_t)(m->IN + m->OUT) * (size_t)n);
   if (!dx) return mfail(m, FVLB_ENOMEM, "fvlb_mlp_infer: device allocation failed");
   float* dy = dx + (size_t)m->IN * n;
   cudaError_t e = cudaMemcpyAsync(dx, x, sizeof(float) * m->IN * n, cudaMemcpyHostToDevice, m->stream);
@@ -801,6 +815,8 @@ int fvlb_mlp_infer(fvlb_mlp_t m, const float* x, long n, float* y) {
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(y, dy, sizeof(float) * m->OUT * n, cudaMemcpyDeviceToHost, m->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
+  else cudaStreamSynchronize(m->stream);
+  stage_give(m, dx);
   if (e != cudaSuccess) return mfail(m, FVLB_ECUDA, std::string("fvlb_mlp_infer: ") + cudaGetErrorString(e));
   return FVLB_OK;
 }
