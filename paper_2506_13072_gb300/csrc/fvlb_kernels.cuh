@@ -140,8 +140,11 @@ __device__ __forceinline__ T* opaque(T* p) {
   return p;
 }
 
-// load f_i(s) (16-bit forms: s_i / KF + e_i(U) with the node's stored U)
-template <class L, class S>
+// load f_i(s) (16-bit forms: s_i / KF + e_i(U) with the node's stored U).
+// BITS: 16-bit values by the builtin load of their bits.  (The headers' __ldg
+// of the 16-bit types are inline assembly, which the compiler keeps in place:
+// better or worse from kernel to kernel, see k_fields.)
+template <class L, class S, bool BITS = false>
 __device__ __forceinline__ void load_f(const S* __restrict__ f, long long pitch,
                                        long long s, RT<S> (&fv)[L::Q]) {
   using R = RT<S>;
@@ -151,8 +154,14 @@ __device__ __forceinline__ void load_f(const S* __restrict__ f, long long pitch,
 #pragma unroll
     for (int a = 0; a < L::D; ++a) u[a] = U[a * pitch + s];
 #pragma unroll
-    for (int i = 0; i < L::Q; ++i)
-      fv[i] = Store<S>::ld(f + i * pitch + s) * R(1.0f / Store<S>::KF) + feq_u<L, R>(i, u);
+    for (int i = 0; i < L::Q; ++i) {
+      R v;
+      if constexpr (BITS)
+        v = Store<S>::cvtb(__ldg(reinterpret_cast<const unsigned short*>(f + i * pitch + s)));
+      else
+        v = Store<S>::ld(f + i * pitch + s);
+      fv[i] = v * R(1.0f / Store<S>::KF) + feq_u<L, R>(i, u);
+    }
   } else {
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) fv[i] = Store<S>::ld(f + i * pitch + s);
@@ -643,7 +652,10 @@ __global__ void k_init(Grid g, S* __restrict__ f, S* __restrict__ h,
 // WHICH: 0 u [N][D], 1 p [N], 2 A [N][C], 3 tau_p [N][C].  Bound by the reads
 // of the populations; one instance per field, so that each reads only what
 // its field needs and keeps its registers for loads in flight (256^3 FP32, p
-// 4.2 / 1.0 ms and A 4.4 / 1.4 ms).
+// 4.2 / 1.0 ms and A 4.4 / 1.4 ms).  16-bit u reads the bits of its values
+// (FP16, us per call: 32^3 43 without, 35 with, 128^3 401 and 339); p, A and
+// the original scheme's u do not (128^3 p 203 without, 287 with, A 691 and
+// 737, the original scheme's u 638 and 649).
 // ---------------------------------------------------------------------------
 // a product that is not contracted into a following sum
 __device__ __forceinline__ float mul_rounded(float a, float b) { return __fmul_rn(a, b); }
@@ -681,7 +693,7 @@ __global__ void __launch_bounds__(128)
       const int x = (int)(s % g.nx);
       const int y = (int)((s / g.nx) % g.ny);
       R fv[Q];
-      load_f<L, S>(f, P, s, fv);
+      load_f<L, S, WHICH == 0 && !ORIG>(f, P, s, fv);
       R F[3];
       body_force<L, R>(ph, x, y, F);
       if constexpr (ORIG) {  // the original scheme: stress divergence in the force
