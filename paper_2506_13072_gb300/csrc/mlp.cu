@@ -147,7 +147,7 @@ struct GradSmem {
   float h2[kMlpH][LD], d2[kMlpH][LD];
   float dy[8][LD];
   float w[LD];                   // sample weights
-  float loss[kGT];
+  double loss[kGT / 32];
 };
 
 __device__ __forceinline__ float4 lds4(const float* p) { return *reinterpret_cast<const float4*>(p); }
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kGT, 3)
     k_mlp_grad(const float* __restrict__ prm, const float* __restrict__ X,
                const float* __restrict__ T, long long count, long long n, int sample_seed,
                long long batch_base, float delta2, float* __restrict__ part,
-               float* __restrict__ part_loss) {
+               double* __restrict__ part_loss) {
   using PP = MlpParams<IN, OUT>;
   constexpr int H = kMlpH;
   extern __shared__ __align__(16) unsigned char grad_smem[];
@@ -188,7 +188,11 @@ __global__ void __launch_bounds__(kGT, 3)
   // weight gradients rows ti + 8 r and columns tk + 16 c
   const int s4 = tid & 7, j4 = tid >> 3;
   const int ti = tid >> 4, tk = tid & 15;
-  float gw2[8][4] = {}, gw1[8] = {}, gw3[4] = {}, gb = 0.f, gb3 = 0.f, loss = 0.f;
+  float gw2[8][4] = {}, gw1[8] = {}, gw3[4] = {}, gb = 0.f, gb3 = 0.f;
+  // FP64 from tile to tile: a block has up to 18 tiles (576 samples of the
+  // largest call), and beside a large residual of one a sum in FP32 loses the
+  // small ones of the others
+  double loss = 0.0;
 
   const long long ntiles = (n + kTS - 1) / kTS;
   for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -290,6 +294,7 @@ __global__ void __launch_bounds__(kGT, 3)
         wgt = 1.f / (tt / float(OUT) + delta2);
       }
       const float scale = 2.0f * wgt / (float(n) * float(OUT));
+      float tl = 0.f;
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
         const int o = o0 + 4 * p;
@@ -297,9 +302,10 @@ __global__ void __launch_bounds__(kGT, 3)
 #pragma unroll 8
         for (int k = 0; k < H; ++k) y += sm.W3[o][k] * sm.h2[k][sp];
         const float r = sr >= 0 && o < OUT ? y - T[sr * OUT + (o < OUT ? o : 0)] : 0.f;
-        loss += wgt * r * r;
+        tl += wgt * r * r;
         sm.dy[o][sp] = scale * r;
       }
+      loss += (double)tl;
     }
     __syncthreads();
     // backward through layer 3 and GELU: dz2 over d2
@@ -379,11 +385,14 @@ __global__ void __launch_bounds__(kGT, 3)
   }
   out[(tid < H ? PP::B1 : PP::B2) + (tid & (H - 1))] = gb;
   if (tid < OUT) out[PP::B3 + tid] = gb3;
-  sm.loss[tid] = loss;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) loss += __shfl_down_sync(0xffffffffu, loss, o);
+  if ((tid & 31) == 0) sm.loss[tid >> 5] = loss;
   __syncthreads();
   if (tid == 0) {
-    float a = 0.f;
-    for (int q = 0; q < kGT; ++q) a += sm.loss[q];
+    double a = sm.loss[0];
+#pragma unroll
+    for (int q = 1; q < kGT / 32; ++q) a += sm.loss[q];
     part_loss[blockIdx.x] = a;
   }
 }
@@ -394,7 +403,7 @@ __global__ void __launch_bounds__(kGT, 3)
 constexpr int kUpdT = 256;
 __global__ void __launch_bounds__(kUpdT)
     k_mlp_update(float* __restrict__ prm, float* __restrict__ mo, float* __restrict__ ve,
-                 const float* __restrict__ part, const float* __restrict__ part_loss, int nblocks,
+                 const float* __restrict__ part, const double* __restrict__ part_loss, int nblocks,
                  int nparam, float* __restrict__ grad, double* __restrict__ loss,
                  double loss_scale, int adam, float lr, float bc1, float bc2) {
   __shared__ float sum[kUpdT / 32][32];
@@ -496,7 +505,8 @@ struct fvlb_mlp_s {
   long long cap = 0, count = 0;
   float *prm = nullptr, *mo = nullptr, *ve = nullptr, *grad = nullptr;
   float *X = nullptr, *T = nullptr;
-  float *part = nullptr, *part_loss = nullptr;
+  float* part = nullptr;
+  double* part_loss = nullptr;
   double* loss = nullptr;
   MlpPacked* packed = nullptr;
   long long adam_t = 0;
@@ -633,7 +643,7 @@ int fvlb_mlp_create(fvlb_mlp_t* out, int lattice, long capacity, unsigned seed) 
   m->X = static_cast<float*>(malloc_dev(m, sizeof(float) * m->IN * capacity));
   m->T = static_cast<float*>(malloc_dev(m, sizeof(float) * m->OUT * capacity));
   m->part = static_cast<float*>(malloc_dev(m, sizeof(float) * m->NP * (size_t)kGradBlocks));
-  m->part_loss = static_cast<float*>(malloc_dev(m, sizeof(float) * kGradBlocks));
+  m->part_loss = static_cast<double*>(malloc_dev(m, sizeof(double) * kGradBlocks));
   m->loss = static_cast<double*>(malloc_dev(m, sizeof(double)));
   m->packed = static_cast<MlpPacked*>(malloc_dev(m, sizeof(MlpPacked)));
   if (!m->prm || !m->mo || !m->ve || !m->grad || !m->X || !m->T || !m->part || !m->part_loss ||
