@@ -301,11 +301,14 @@ __device__ __forceinline__ void fused_tile(
     if (has && mm >= 0) {
       const uint32_t s = node_of(mm, gx, gy);
 #pragma unroll
-      for (int i = 1; i < Q; ++i) v.f[i] = b.f_in[(uint32_t)i * P32 + s];
+      for (int i = 1; i < Q; ++i) {
+        if constexpr (V2) v.f[i] = ld_state(b.f_in + ((uint32_t)i * P32 + s));
+        else v.f[i] = b.f_in[(uint32_t)i * P32 + s];
+      }
       if constexpr (V2) {
         const float* U = f_ext<L>(b.f_in, P);
 #pragma unroll
-        for (int a = 0; a < D; ++a) v.u[a] = __ldg(U + ((uint32_t)a * P32 + s));
+        for (int a = 0; a < D; ++a) v.u[a] = ld_state(U + ((uint32_t)a * P32 + s));
       }
     }
   };
@@ -400,10 +403,10 @@ __device__ __forceinline__ void fused_tile(
             const uint32_t* fw = reinterpret_cast<const uint32_t*>(b.f_in);
             const float* U = f_ext<L>(b.f_in, P);
 #pragma unroll
-            for (int i = 1; i < Q; ++i) v.f[i] = __ldg(fw + (((uint32_t)i * P32 + s0) >> 1));
+            for (int i = 1; i < Q; ++i) v.f[i] = ld_state(fw + (((uint32_t)i * P32 + s0) >> 1));
 #pragma unroll
             for (int a = 0; a < D; ++a)
-              v.u[a] = __ldg(reinterpret_cast<const float2*>(U + ((uint32_t)a * P32 + s0)));
+              v.u[a] = ld_state(reinterpret_cast<const float2*>(U + ((uint32_t)a * P32 + s0)));
           }
         };
         auto pstore = [&](int mm, int q, const Pair& v) {
