@@ -110,7 +110,7 @@ __global__ void k_closure_pairs(Grid g, Phys<RT<S>> ph, const S* __restrict__ f,
 // start in different banks.
 // 32768 samples in 3D, a call of fvlb_mlp_grad from host arrays: 310 us with
 // one thread per sample, 125 us now; of these this kernel 50 us (10.7 TFMA/s,
-// 37 % of the FMA pipe: shared-memory latency at 12 warps an SM, and 2.25
+// 27 % of the FMA pipe's 40.3: shared-memory latency at 12 warps an SM, and 2.25
 // tiles a block on average where some have 3) and the sum of the partials 10.
 // ---------------------------------------------------------------------------
 
@@ -146,7 +146,6 @@ struct GradSmem {
   float h1[kMlpH][LD], d1[kMlpH][LD];   // activations; GELU derivatives, then dz
   float h2[kMlpH][LD], d2[kMlpH][LD];
   float dy[8][LD];
-  float w[LD];                   // sample weights
   double loss[kGT / 32];
 };
 
@@ -165,8 +164,7 @@ template <int IN, int OUT>
 __global__ void __launch_bounds__(kGT, 3)
     k_mlp_grad(const float* __restrict__ prm, const float* __restrict__ X,
                const float* __restrict__ T, long long count, long long n, int sample_seed,
-               long long batch_base, float delta2, float* __restrict__ part,
-               double* __restrict__ part_loss) {
+               float delta2, float* __restrict__ part, double* __restrict__ part_loss) {
   using PP = MlpParams<IN, OUT>;
   constexpr int H = kMlpH;
   extern __shared__ __align__(16) unsigned char grad_smem[];
@@ -202,11 +200,10 @@ __global__ void __launch_bounds__(kGT, 3)
     if (tid < kTS) {
       const long long off = tile * kTS + tid;
       if (off < n) {
-        const long long gi = batch_base + off;
         src = sample_seed >= 0
-                  ? (long long)(((uint64_t)mix32((uint32_t)gi * 0x9e3779b9u ^ mix32((uint32_t)sample_seed)) *
+                  ? (long long)(((uint64_t)mix32((uint32_t)off * 0x9e3779b9u ^ mix32((uint32_t)sample_seed)) *
                                  (uint64_t)count) >> 32)
-                  : gi;
+                  : off;
       }
 #pragma unroll
       for (int k = 0; k < 16; ++k) sm.x[k][tid] = src >= 0 && k < IN ? X[src * IN + k] : 0.f;
@@ -280,11 +277,10 @@ __global__ void __launch_bounds__(kGT, 3)
       const long long off = tile * kTS + sp;
       long long sr = -1;
       if (off < n) {
-        const long long gi = batch_base + off;
         sr = sample_seed >= 0
-                 ? (long long)(((uint64_t)mix32((uint32_t)gi * 0x9e3779b9u ^ mix32((uint32_t)sample_seed)) *
+                 ? (long long)(((uint64_t)mix32((uint32_t)off * 0x9e3779b9u ^ mix32((uint32_t)sample_seed)) *
                                 (uint64_t)count) >> 32)
-                 : gi;
+                 : off;
       }
       // sample weight: 1, or 1 / (mean_o t_o^2 + delta^2) for the relative loss
       float wgt = 1.f;
@@ -580,7 +576,7 @@ cudaError_t launch_grad_of(fvlb_mlp_t m, const float* X, const float* T, long lo
   auto kern = k_mlp_grad<IN, OUT>;
   const cudaError_t e = allow_dynamic_smem(kern, sm);
   if (e != cudaSuccess) return e;
-  kern<<<grad_blocks(n), kGT, sm, m->stream>>>(m->prm, X, T, count, n, seed, 0, d2, m->part,
+  kern<<<grad_blocks(n), kGT, sm, m->stream>>>(m->prm, X, T, count, n, seed, d2, m->part,
                                                m->part_loss);
   return cudaGetLastError();
 }
