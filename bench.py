@@ -270,13 +270,21 @@ def run_reference(args, rank, world):
     print(json.dumps(line), flush=True)
 
 
-def kernel_label(lattice: str, precision: str) -> str:
-    """The fused-step kernel instance the library launches for this workload."""
+def kernel_label(lattice: str, precision: str, n: int, sms: int,
+                 original: bool = False) -> str:
+    """The fused-step kernel instance the library launches for a periodic n^2
+    or n^3 grid with n a multiple of its wide tile and several waves of them
+    (where the rows or the waves leave wide tiles half empty it may take tiles
+    of one warp, and where n is off the 16-byte grid padded ones, which this
+    does not follow).  MINB: the blocks per SM, plus 100 times the stage buffers
+    where they are not three."""
     S = {"fp64": "double", "fp32": "float", "fp16_dev": "__half", "bf16_dev": "__nv_bfloat16",
          "fp16_dev_sr": "half_sr", "bf16_dev_sr": "bf16_sr"}[precision]
     wide, half = precision == "fp64", precision not in ("fp64", "fp32")
     if lattice == "d2q9":
         gx, kg, minb = (2, 1, 3) if wide else ((4, 1, 4) if half else (4, 1, 2))
+        if precision == "fp32" and not original and n * n > sms * minb * 32 * 32 * gx:
+            minb += 400
         slots, lat = 32 * gx + 2, "D2Q9"
     else:
         gx, kg, minb = (1, 2, 2) if wide else ((2, 2, 3) if half else (2, 2, 2))
@@ -449,7 +457,9 @@ def run_ours(args, rank, world, dist):
                      "traffic": tr["dram_bytes_per_launch"] if tr else None,
                      "algorithmic_bytes_per_launch": bpu * sites,
                      "bytes_per_update": bpu, "peak_source": f"{which} hbm_gbs (copy)",
-                     "kernel": kernel_label(args.lattice, args.precision)
+                     "kernel": kernel_label(args.lattice, args.precision, pr.nx,
+                                            torch.cuda.get_device_properties(0).multi_processor_count,
+                                            original=launches != 1)
                                + ("" if launches == 1 else
                                   "; original scheme: k_taup + k_fdiv + this kernel "
                                   "(ORIG) per step, state bytes over the step time")},
@@ -508,7 +518,7 @@ def form_rate(F, pr, precision, steps, warmup, stream, kernel=0, scheme=0):
 
 def batch_rate(F, precision, stream, steps=40):
     """512 uneven D2Q9 instances (four-roll / Poiseuille, n log-uniform in
-    [32, 512], seed 0) in one persistent launch per step, graph-replayed,
+    [32, 512], seed 0) in one launch per step, graph-replayed,
     tile shape autotuned (the tuning steps run before the timed region)."""
     import torch
 
