@@ -283,7 +283,7 @@ int build_graph(fvlb_batch_t b) {
     d.maps = b->maps + (size_t)d.parity * b->count;
     d.first = 0;
     if (e == cudaSuccess) e = batch_step(d);
-    }
+  }
   cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
   if (e == cudaSuccess) e = e2;
   if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph, g, 0);

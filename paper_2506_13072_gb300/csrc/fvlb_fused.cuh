@@ -1127,11 +1127,13 @@ __global__ void __launch_bounds__(FusedShape<L, S, GX, KG, CL>::NT, blocks_of(MI
   StagePos pos;
   fused_tile<L, S, GX, KG, MINB, WALLS, PADDED, CL, ORIG>(sm, g, ph, b, mchunk, blockIdx.x,
                                                       blockIdx.y, blockIdx.z, &tm, tm.on != 0, pos);
-  // The next step's blocks may come in when every block's first collision warp
-  // is through.  (Earlier, they take the free slots of SMs that are busy with
-  // this step: 64^2 FP64 17.3 us a step with the trigger at the start, 11.1
-  // at the last plane, 11.0 here, 12.3 without; 128^2 FP32 3.75, 3.67, 3.12
-  // and 6.15; 517 x 333 FP32 11.2, 11.0, 10.8 and 12.5; large grids the same.)
+  // The next step's blocks may come in when every block's collision warps are
+  // through (an exit counts as well: without the call the times are the same).
+  // Earlier, they take the free slots of SMs that are busy with this step: 64^2
+  // FP64 12.6 us a step with the trigger at the start, 6.3 at the last plane,
+  // 6.1 here, 8.2 without the programmatic edge; 128^2 FP32 3.25, 2.96, 2.57
+  // and 4.10; 517 x 333 FP32 10.6, 10.3, 10.05 and 12.3; 128^3 FP32 360.6 to
+  // 362.0 and 363.8.
   if (threadIdx.x < FusedShape<L, S, GX, KG, CL>::NCW * 32) pdl_trigger();
 }
 

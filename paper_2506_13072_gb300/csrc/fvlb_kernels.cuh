@@ -30,8 +30,9 @@ template <class S>
 using RT = typename Store<S>::R;
 
 // Bulk tensor copies (TMA) into shared memory, completed on an mbarrier.
-// A warp's lane 0 arms the barrier with the byte count of its copies and
-// issues them; every lane of the warp waits for the barrier's phase.
+// One thread of the block arms the barrier with the byte count of a buffer's
+// copies and issues them; every warp that reads the buffer waits for the
+// barrier's phase.
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }

@@ -165,6 +165,14 @@ cudaError_t allow_dynamic_smem(K* kern, size_t bytes) {
 //   D2Q9 FP32 4,1,2: 20270 (18102); KG 3: 18223, GX 2: 19012
 //   D2Q9 FP16 4,1,4: 28200 (14835); MINB 3: 27000, 5: 23800, GX 2: 23520
 //   D2Q9 FP64 (512^2) 2,1,3: 2110 (948); KG 3: 1463, GX 4: 1968
+// With stochastic rounding 2,2,3 and 4,1,4 as well (us a step, the kernel with
+// one thread per stress component and now: 128^3 FP16 625 / 510, BF16
+// 556 / 424; 1024^2 FP16 94 / 57, BF16 90 / 52).
+// Spills that these budgets cost (bytes stored / loaded per thread): D3Q19
+// 16-bit 24 / 24 to 28 / 28 at 80 registers, 24 / 24 to 44 / 44 with
+// stochastic rounding (MINB 2 leaves 128 registers and is slower at 128^3, see
+// above); D2Q9 FP64 up to 92 / 80 at 128 registers, 160 / 104 in the original
+// scheme; D2Q9 16-bit with stochastic rounding 8 / 8.
 // SMALL: one warp's nodes per tile, for grids that leave the chip idle
 // otherwise (the larger KG spreads FP64 over the four quarters of an SM; 32^3
 // FP32 1,2,4 6.9 us a step, 1,2,3 8.2, the wide tile 11.7; 48^3 FP16 1,2,5
@@ -187,9 +195,9 @@ struct StepShape {
 //  - More: all planes and the prologues' work (`pro` planes a block) at the
 //    full SM's rate, and a share of one block's time for the uneven end.
 // us per step, this rule and the one before it (the fewest planes that still
-// fill the last wave, 2.5 planes a prologue): 64^2 FP64 6.2 / 10.2, 8x128
-// FP32 2.3 / 2.6, 100^3 FP32 215 / 223, 161x97x65 234 / 253, 64^3 FP64
-// 476 / 519, 128^3 FP16 348 / 356.
+// fill the last wave, 2.5 planes a prologue), both with the present kernels:
+// 64^2 FP64 6.1 / 10.2, 8x128 FP32 2.2 / 2.6, 100^3 FP32 208 / 216, 161x97x65
+// 226 / 245, 64^3 FP64 467 / 501, 128^3 FP16 297 / 298.
 struct ChunkModel {
   double slope, lat, pro, tail;
 };
@@ -309,9 +317,11 @@ cudaError_t fused_step(const StepDesc& d, const Grid& g, const Phys<RT<S>>& ph,
     if (small)
       return launch_fused<L, S, true, Small::GX, Small::KG, Small::MINB, false, ORIG>(d, g, ph, b);
   }
-  // D2Q9 FP32 with several waves of blocks: a fourth stage buffer (2048^2
-  // 206.9 us a step, 215.6 with three, 209.4 with five; with one wave it costs:
-  // 512^2 11.9 against 11.6, 517x333 10.5 against 10.1; 16-bit storage 5 %)
+  // D2Q9 FP32 with more than one wave of 32-row chunks (1.25 M nodes): a fourth
+  // stage buffer.  us a step with four and three, constant force: 512^2 11.2 and 10.9, 1024^2
+  // 53.3 and 53.1, 1120^2 68.2 and 69.6, 1280^2 83.7 and 86.2, 1536^2 118.7 and
+  // 121.9, 1733x1337 121.5 and 122.9, 2048^2 201.8 and 210.0 (a fifth costs 1 %
+  // there; with 16-bit storage the fourth costs 5 %)
   if constexpr (L::D == 2 && std::is_same<S, float>::value && !ORIG) {
     if ((long long)d.nx * d.ny > (long long)d.sms * Big::MINB * 32 * 32 * Big::GX)
       return launch_fused<L, S, false, Big::GX, Big::KG, 400 + Big::MINB, false, ORIG>(d, g, ph, b);
