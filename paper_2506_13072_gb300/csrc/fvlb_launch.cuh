@@ -318,10 +318,10 @@ cudaError_t fused_step(const StepDesc& d, const Grid& g, const Phys<RT<S>>& ph,
       return launch_fused<L, S, true, Small::GX, Small::KG, Small::MINB, false, ORIG>(d, g, ph, b);
   }
   // D2Q9 FP32 with more than one wave of 32-row chunks (1.25 M nodes): a fourth
-  // stage buffer.  us a step with four and three, constant force: 512^2 11.2 and 10.9, 1024^2
-  // 53.3 and 53.1, 1120^2 68.2 and 69.6, 1280^2 83.7 and 86.2, 1536^2 118.7 and
-  // 121.9, 1733x1337 121.5 and 122.9, 2048^2 201.8 and 210.0 (a fifth costs 1 %
-  // there; with 16-bit storage the fourth costs 5 %)
+  // stage buffer.  us a step with four and three, constant force: 512^2 11.2
+  // and 10.9, 1024^2 53.3 and 53.1, 1120^2 68.2 and 69.6, 1280^2 83.7 and 86.2,
+  // 1536^2 118.7 and 121.9, 1733x1337 121.5 and 122.9, 2048^2 201.8 and 210.0
+  // (a fifth costs 1 % there; with 16-bit storage the fourth costs 5 %)
   if constexpr (L::D == 2 && std::is_same<S, float>::value && !ORIG) {
     if ((long long)d.nx * d.ny > (long long)d.sms * Big::MINB * 32 * 32 * Big::GX)
       return launch_fused<L, S, false, Big::GX, Big::KG, 400 + Big::MINB, false, ORIG>(d, g, ph, b);
